@@ -399,7 +399,7 @@ def topk_runs_delete_min_flexible(ctx: Context, keys, run_off, cursor, kmin: int
 def topk_select_kth(ctx: Context, keys, k: int, params: topk_params | None = None, stream=None, out=None,
                     check: bool = True):
     """The key of rank k and its position (the k-th smallest, or the k-th
-    largest with TOPK_FLAG_LARGEST); the selected set stays in the context.
+    largest with TOPK_FLAG_LARGEST), without the selected set.
     Returns (kth_key[1] of the key dtype, kth_idx[1] uint32)."""
     torch = _torch()
     if out is None:

@@ -218,6 +218,7 @@ struct SelArgs {
     u32* pass_done;           // block-done counter of the pass (zero between passes)
     u32 samp_cap;
     int first_dense;          // first level's pass mode chosen by the host (0/1), or -1
+    u32 kth_only;             // only the rank-k pair is wanted: no selected element is written
 };
 
 

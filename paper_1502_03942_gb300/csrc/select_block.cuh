@@ -109,7 +109,7 @@ __device__ void run_pass_to(const SelArgs& a, const SelState& s, u64 tile0, u64 
     sink.out_keys = static_cast<raw_t*>(a.out_keys);
     sink.out_idx = a.out_idx;
     sink.out_base = s.out_base;
-    sink.cap_a = s.k_rem;
+    sink.cap_a = a.kth_only ? 0 : s.k_rem;
     sink.ck = static_cast<key_t*>(a.cand_key[s.dst - 1]);
     sink.ci = a.cand_idx[s.dst - 1];
     sink.cap_b = a.cap_b;
@@ -258,10 +258,10 @@ template <int DT, class SM> __device__ void block_finish(const SelArgs& a, SM& s
         return;
     }
     const ct kth = block_select_hist<KW, NT>(sm.samp, count, lo, hi, (u32)(s.k_rem - 1), sm.hs);
-    if (threadIdx.x == 0) sm.kept = 0;
+    if (threadIdx.x == 0) sm.kept = a.kth_only ? (u32)s.k_rem : 0u;
     __syncthreads();
     raw_t* ok_out = static_cast<raw_t*>(a.out_keys);
-    for (u32 base = 0; base < count; base += NT * U) {
+    for (u32 base = 0; base < count && !a.kth_only; base += NT * U) {
         u32 selm = 0;
 #pragma unroll
         for (int u = 0; u < U; ++u) {

@@ -297,7 +297,7 @@ template <int DT> struct Sink {
     raw_t* out_keys;
     u32* out_idx;
     u64 out_base; // first free output slot
-    u64 cap_a;    // slots available to this pass (k_rem)
+    u64 cap_a;    // slots available to this pass (k_rem; 0: a is counted and not written)
     key_t* ck;
     u32* ci;
     u64 cap_b;
@@ -622,7 +622,7 @@ __device__ __forceinline__ void classify_emit(const KeyT (&kk)[16], PosF pos, u3
     u64 ra = sm.ba[warp], rb = sm.bb[warp];
     const u32 below = lanemask_lt();
     typedef typename Key<DT>::raw_t raw_t;
-    if (HAS_A && __any_sync(0xffffffffu, ma)) {
+    if (HAS_A && sink.cap_a != 0 && __any_sync(0xffffffffu, ma)) {
         if (ra + wa <= sink.cap_a) { // the warp's run fits: no per-element bound
             raw_t* okp = sink.out_keys + sink.out_base + ra;
             u32* oip = sink.out_idx + sink.out_base + ra;
@@ -741,7 +741,7 @@ __device__ __forceinline__ void lq_write(const typename Comp<Key<DT>::KW>::key_t
             isb = c >= pl && c <= pr;
         }
         const u32 bala = __ballot_sync(0xffffffffu, isa), balb = __ballot_sync(0xffffffffu, isb);
-        if (isa) sink.put_a(ba + __popc(bala & below), kv, iv);
+        if (isa) sink.put_a(ba + __popc(bala & below), kv, iv); // (writes nothing where cap_a = 0)
         if (isb) sink.put_b(bb + __popc(balb & below), kv, iv);
         ba += __popc(bala);
         bb += __popc(balb);

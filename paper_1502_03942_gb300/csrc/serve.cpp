@@ -66,7 +66,7 @@ struct Slot {
 uint64_t slot_held(const Slot& slot) {
     const topk_ctx* c = slot.ctx;
     if (!c) return 0;
-    return (uint64_t)c->scratch.bytes + c->freq.bytes + c->aux.bytes + CTX_FIXED_BYTES + 52ull * MAX_BATCH_ROWS;
+    return (uint64_t)c->scratch.bytes + c->freq.bytes + CTX_FIXED_BYTES + 52ull * MAX_BATCH_ROWS;
 }
 
 uint64_t request_bytes(const topk_request& r) {
