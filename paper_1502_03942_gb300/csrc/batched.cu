@@ -227,7 +227,6 @@ __device__ __forceinline__ SelArgs row_args(const BatchArgs& b, u32 row, u64 r0,
     a.parts = b.parts;
     a.sample = b.sample;
     a.finish_T = b.finish_T;
-    a.grid_G = b.finish_T;
     a.z = b.z;
     a.flags = b.flags;
     a.aligned = 0;
@@ -634,8 +633,7 @@ __global__ void __launch_bounds__(NT, (BatchVariant<Key<DT>::KW, NT>::MINB)) k_b
         a.parts = b.parts;
         a.sample = b.sample;
         a.finish_T = b.finish_T;
-        a.grid_G = b.finish_T;
-        a.z = b.z;
+            a.z = b.z;
         a.flags = b.flags;
         a.aligned = 0;
         a.err = b.err;
@@ -704,14 +702,14 @@ static topk_status launch_batched(topk_ctx* ctx, const BatchArgs& b, cudaStream_
     if (rs != TOPK_OK) return rs;
     int pass_per_sm = 1, plan_per_sm = 1;
     if (b.split != WIDE_NONE && (rs = wide_setup<DT>(ctx->device, pass_per_sm, plan_per_sm)) != TOPK_OK) return rs;
-    cudaError_t e = launch_dep(k_batch_order, 1, 1024, 0, st, b);
+    cudaError_t e = launch_dep(k_batch_order, 1, 1024, 0, st, 1, b);
     if (e == cudaSuccess && b.split != WIDE_NONE) {
-        e = launch_dep(k_wide_plan<DT>, ctx->sms * plan_per_sm, WIDE_PLAN_NT, sizeof(BatchSmem<KW, WIDE_PLAN_NT>), st,
+        e = launch_dep(k_wide_plan<DT>, ctx->sms * plan_per_sm, WIDE_PLAN_NT, sizeof(BatchSmem<KW, WIDE_PLAN_NT>), st, 1,
                        b);
         if (e == cudaSuccess)
-            e = launch_dep(k_wide_pass<DT>, ctx->sms * pass_per_sm, WIDE_NT, WideCfg<DT>::SMEM, st, b);
+            e = launch_dep(k_wide_pass<DT>, ctx->sms * pass_per_sm, WIDE_NT, WideCfg<DT>::SMEM, st, 1, b);
     }
-    if (e == cudaSuccess) e = launch_dep(k_batched<DT, NT>, ctx->sms * per_sm, NT, sizeof(BatchSmem<KW, NT>), st, b);
+    if (e == cudaSuccess) e = launch_dep(k_batched<DT, NT>, ctx->sms * per_sm, NT, sizeof(BatchSmem<KW, NT>), st, 1, b);
     if (e != cudaSuccess) return cuda_status(e);
     count_launch(ctx, b.split != WIDE_NONE ? 4 : 2);
     return cuda_status(cudaGetLastError());

@@ -191,6 +191,16 @@ __device__ __forceinline__ int bit_length_fast(u128 v) {
     return hi ? 128 - __clzll((long long)hi) : bit_length_fast((u64)v);
 }
 
+// The first level's candidates are also counted over equal bins of its
+// bracket: bin (packed composite - base) >> shift.
+constexpr u32 HB_BITS = 11;
+constexpr u32 HB_BINS = 1u << HB_BITS;
+struct alignas(16) LevelBins {
+    u32 h[HB_BINS];
+    u128 base;
+    u32 shift;
+};
+
 // Arguments common to every kernel of one topk_select call.
 struct SelArgs {
     const void* keys;         // input (raw keys)
@@ -207,16 +217,14 @@ struct SelArgs {
     u32 parts;                // sampling partitions
     u32 sample;               // draws per level
     u32 finish_T;             // single-block finish threshold
-    u32 grid_G;               // grid levels run while m_src > G
     float z;                  // pivot margin factor
     u32 flags;
     u32 aligned;              // input is 16-byte aligned
     u32* err;                 // context's latched error word
-    // grid-level sampling (k_sample / k_pivots) and the end-of-pass branch
-    void* samp;               // sample composites, capacity samp_cap
-    u32* samp_count;          // number drawn into samp (zero between levels)
     u32* pass_done;           // block-done counter of the pass (zero between passes)
-    u32 samp_cap;
+    LevelBins* bins;          // the first level's bins (set up by k_plan), or null
+    u32 idx_bits;             // bits that hold every position below n
+    u32 list_max;             // undecided elements that the finish takes without a second pass
     int first_dense;          // first level's pass mode chosen by the host (0/1), or -1
     u32 kth_only;             // only the rank-k pair is wanted: no selected element is written
 };

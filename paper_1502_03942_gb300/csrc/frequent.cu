@@ -565,7 +565,7 @@ topk_status topk_frequent(topk_ctx* ctx, const void* d_objects, uint64_t n, topk
     const u64 tile_objs = (u64)FQ_NT * FQ_QUADS * 4;
     const u64 tiles = (n + tile_objs - 1) / tile_objs;
     const int grid = (int)std::max<u64>(1, std::min<u64>(tiles, (u64)ctx->sms * std::max(per_sm, 1)));
-    e = launch_dep(kern, grid, FQ_NT, sizeof(FqLocal), st, a);
+    e = launch_dep(kern, grid, FQ_NT, sizeof(FqLocal), st, 1, a);
     if (e != cudaSuccess) return cuda_status(e);
     count_launch(ctx);
 
@@ -573,14 +573,14 @@ topk_status topk_frequent(topk_ctx* ctx, const void* d_objects, uint64_t n, topk
     rs = topk_select(ctx, table, cap, need, TOPK_U64, sel, sel_idx, kth, kth_idx, nullptr, stream);
     if (rs != TOPK_OK) return rs;
     if (!ec) {
-        e = launch_dep(k_freq_decode, (int)((fp->k + 255) / 256), 256, 0, st, (const u64*)sel, (const u64*)kth,
+        e = launch_dep(k_freq_decode, (int)((fp->k + 255) / 256), 256, 0, st, 1, (const u64*)sel, (const u64*)kth,
                        fp->k, d_out_obj, d_out_count, ctx->d_err, (const u64*)cursor,
                        (u64)n, d_sample_size);
         count_launch(ctx);
         return cuda_status(e);
     }
     // 3. EC: exact recount of the k* candidates (Section 7.2)
-    e = launch_dep(k_freq_check, 1, 32, 0, st, (const u64*)kth, ctx->d_err);
+    e = launch_dep(k_freq_check, 1, 32, 0, st, 1, (const u64*)kth, ctx->d_err);
     u32* exact = reinterpret_cast<u32*>(base + o_exact);
     if (e == cudaSuccess) e = cudaMemsetAsync(exact, 0, 4ull * kstar, st);
     if (e != cudaSuccess) return cuda_status(e);
@@ -614,10 +614,10 @@ topk_status topk_frequent(topk_ctx* ctx, const void* d_objects, uint64_t n, topk
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_x, ek, FQ_NT, smem);
     const u64 quad_blocks = ((n + 3) / 4 + (u64)FQ_NT * FQ_XQUADS - 1) / ((u64)FQ_NT * FQ_XQUADS);
     const int grid_x = (int)std::max<u64>(1, std::min<u64>(quad_blocks, (u64)ctx->sms * std::max(per_sm_x, 1)));
-    e = launch_dep(ek, grid_x, FQ_NT, smem, st, x);
+    e = launch_dep(ek, grid_x, FQ_NT, smem, st, 1, x);
     u64* comp = reinterpret_cast<u64*>(base + o_comp);
     if (e == cudaSuccess)
-        e = launch_dep(k_freq_compose, (int)((kstar + 255) / 256), 256, 0, st, (const u64*)sel, (const u32*)exact,
+        e = launch_dep(k_freq_compose, (int)((kstar + 255) / 256), 256, 0, st, 1, (const u64*)sel, (const u32*)exact,
                        kstar, comp);
     if (e != cudaSuccess) return cuda_status(e);
     count_launch(ctx, 3);
@@ -628,7 +628,7 @@ topk_status topk_frequent(topk_ctx* ctx, const void* d_objects, uint64_t n, topk
     u32* kth2_idx = reinterpret_cast<u32*>(base + o_kth2 + 8);
     rs = topk_select(ctx, comp, kstar, fp->k, TOPK_U64, sel2, idx2, kth2, kth2_idx, nullptr, stream);
     if (rs != TOPK_OK) return rs;
-    e = launch_dep(k_freq_decode, (int)((fp->k + 255) / 256), 256, 0, st, (const u64*)sel2, (const u64*)kth2, fp->k,
+    e = launch_dep(k_freq_decode, (int)((fp->k + 255) / 256), 256, 0, st, 1, (const u64*)sel2, (const u64*)kth2, fp->k,
                    d_out_obj, d_out_count, ctx->d_err, (const u64*)cursor, (u64)n,
                    d_sample_size);
     count_launch(ctx);

@@ -680,11 +680,11 @@ static topk_status run_sorted_runs(topk_ctx* ctx, const void* d_keys, const uint
     // a flexible search usually ends within a round or two (each trial lands
     // in the range with constant probability); the spare rounds return at once
     const u32 rounds = flexible ? std::min<u32>(runs_rounds_for(p, kmax, a.d), 4u) : runs_rounds_for(p, k, a.d);
-    cudaError_t e = launch_dep(k_runs_init, 1, RUN_FIN_NT, 0, st, a);
+    cudaError_t e = launch_dep(k_runs_init, 1, RUN_FIN_NT, 0, st, 1, a);
     if (e == cudaSuccess && (prm.flags & TOPK_FLAG_CHECK_SORTED))
-        e = launch_dep(k_runs_check_sorted, (int)p, RUN_NT, 0, st, a);
-    for (u32 r = 0; r < rounds && e == cudaSuccess; ++r) e = launch_dep(k_runs_round, (int)a.d, RUN_NT, 0, st, a);
-    if (e == cudaSuccess) e = launch_dep(k_runs_finish, 1, RUN_FIN_NT, fin_smem, st, a);
+        e = launch_dep(k_runs_check_sorted, (int)p, RUN_NT, 0, st, 1, a);
+    for (u32 r = 0; r < rounds && e == cudaSuccess; ++r) e = launch_dep(k_runs_round, (int)a.d, RUN_NT, 0, st, 1, a);
+    if (e == cudaSuccess) e = launch_dep(k_runs_finish, 1, RUN_FIN_NT, fin_smem, st, 1, a);
     if (e != cudaSuccess) return cuda_status(e);
     count_launch(ctx, 2 + rounds + ((prm.flags & TOPK_FLAG_CHECK_SORTED) ? 1 : 0));
     return cuda_status(cudaGetLastError());

@@ -353,6 +353,28 @@ template <int DT> struct Sink {
     }
 };
 
+// Counts of the b elements over equal bins of the bracket, kept by a pass
+// while it emits them (in shared memory; added to the grid's bins when the
+// block is done), so that the next level's pivots can be read off exact counts
+// instead of a new sample.  The position takes only `bn` bits of the packed
+// composite, so that the bins of a bracket of few distinct keys are not spent on
+// positions that no element has.
+struct NoBins {
+    template <class K> __device__ __forceinline__ void add(K, u32) const {}
+};
+template <int KW> struct BinHist {
+    typedef typename Comp<KW>::t ct;
+    u32* h;
+    ct base;
+    u32 sh, bn;
+    __device__ __forceinline__ void add(typename Comp<KW>::key_t k, u32 x) const {
+        if (!h) return; // the candidates are expected to fit the finish
+        const ct c = ((ct)k << bn) | x;
+        const ct d = c > base ? (ct)((c - base) >> sh) : (ct)0;
+        atomicAdd(&h[d < (ct)HB_BINS ? (u32)d : HB_BINS - 1], 1u);
+    }
+};
+
 // ---------------------------------------------- bounds on raw key bits
 // Whether image(x) <= T (or >= T) for the order-preserving image of a key
 // type, decided by one integer comparison of the raw bits x against a bound
@@ -557,9 +579,9 @@ template <int ID, int N> struct SyncNamed {
 // is classified exactly on the full (key, position) pair; any other key is in
 // c.  So most elements cost one subtraction and one comparison.  EXACT
 // classifies every element on the pair (used when lo > 0, a narrowed window).
-template <int NT, bool HAS_A, bool EXACT, class Sync, int DT, class CT, class KeyT, class PosF>
+template <int NT, bool HAS_A, bool EXACT, class Sync, int DT, class CT, class KeyT, class PosF, class Bins = NoBins>
 __device__ __forceinline__ void classify_emit(const KeyT (&kk)[16], PosF pos, u32 valid, CT lo, CT pl, CT pr,
-                                              const Sink<DT>& sink, PassSmem<NT>& sm) {
+                                              const Sink<DT>& sink, PassSmem<NT>& sm, const Bins& bins = Bins{}) {
     typedef Comp<Key<DT>::KW> C;
     const u32 warp = threadIdx.x >> 5, lane = lane_id();
     u32 ma = 0, mb = 0;
@@ -663,6 +685,7 @@ __device__ __forceinline__ void classify_emit(const KeyT (&kk)[16], PosF pos, u3
                 if (bit) {
                     bkp[r] = kk[s];
                     bip[r] = x;
+                    bins.add(kk[s], x);
                 }
                 const u32 c = (u32)__popc(bal);
                 bkp += c;
@@ -672,7 +695,10 @@ __device__ __forceinline__ void classify_emit(const KeyT (&kk)[16], PosF pos, u3
 #pragma unroll
             for (int s = 0; s < 16; ++s) {
                 const u32 bal = __ballot_sync(0xffffffffu, (mb >> s) & 1u);
-                if ((mb >> s) & 1u) sink.put_b(rb + __popc(bal & below), kk[s], pos(s));
+                if ((mb >> s) & 1u) {
+                    sink.put_b(rb + __popc(bal & below), kk[s], pos(s));
+                    bins.add(kk[s], pos(s));
+                }
                 rb += __popc(bal);
             }
         }
@@ -720,10 +746,11 @@ struct LQState {
     __device__ static LQState make() { return LQState{0u, 0u, 0u, 0u, 0ull, 0ull}; }
 };
 
-template <int DT>
+template <int DT, class Bins>
 __device__ __forceinline__ void lq_write(const typename Comp<Key<DT>::KW>::key_t* qk, const u32* qi, u32 cnt, u32 mx,
                                          u64 ra, u64 rb, const Sink<DT>& sink, typename Comp<Key<DT>::KW>::t lo,
-                                         typename Comp<Key<DT>::KW>::t pl, typename Comp<Key<DT>::KW>::t pr) {
+                                         typename Comp<Key<DT>::KW>::t pl, typename Comp<Key<DT>::KW>::t pr,
+                                         const Bins& bins) {
     typedef Comp<Key<DT>::KW> C;
     typedef typename C::t ct;
     u64 ba = __shfl_sync(0xffffffffu, (unsigned long long)ra, 0);
@@ -742,20 +769,24 @@ __device__ __forceinline__ void lq_write(const typename Comp<Key<DT>::KW>::key_t
         }
         const u32 bala = __ballot_sync(0xffffffffu, isa), balb = __ballot_sync(0xffffffffu, isb);
         if (isa) sink.put_a(ba + __popc(bala & below), kv, iv); // (writes nothing where cap_a = 0)
-        if (isb) sink.put_b(bb + __popc(balb & below), kv, iv);
+        if (isb) {
+            sink.put_b(bb + __popc(balb & below), kv, iv);
+            bins.add(kv, iv);
+        }
         ba += __popc(bala);
         bb += __popc(balb);
     }
 }
 
-template <int DT>
+template <int DT, class Bins>
 __device__ __forceinline__ void lq_flush(WarpQ<Key<DT>::KW>& q, LQState& qs, const Sink<DT>& sink,
                                          typename Comp<Key<DT>::KW>::t lo, typename Comp<Key<DT>::KW>::t pl,
-                                         typename Comp<Key<DT>::KW>::t pr) {
+                                         typename Comp<Key<DT>::KW>::t pr, const Bins& bins) {
     typedef Comp<Key<DT>::KW> C;
     typedef typename C::t ct;
     __syncwarp();
-    if (qs.pmax) lq_write<DT>(q.k[qs.cq ^ 1u], q.i[qs.cq ^ 1u], qs.pcnt, qs.pmax, qs.ra, qs.rb, sink, lo, pl, pr);
+    if (qs.pmax) lq_write<DT>(q.k[qs.cq ^ 1u], q.i[qs.cq ^ 1u], qs.pcnt, qs.pmax, qs.ra, qs.rb, sink, lo, pl, pr,
+                                 bins);
     const u32 lane = lane_id();
     const u32 mx = __reduce_max_sync(0xffffffffu, qs.cnt);
     u32 ca = 0, cb = 0;
@@ -780,12 +811,13 @@ __device__ __forceinline__ void lq_flush(WarpQ<Key<DT>::KW>& q, LQState& qs, con
     __syncwarp();
 }
 
-template <int DT>
+template <int DT, class Bins = NoBins>
 __device__ __forceinline__ void lq_drain(WarpQ<Key<DT>::KW>& q, LQState& qs, const Sink<DT>& sink,
                                          typename Comp<Key<DT>::KW>::t lo, typename Comp<Key<DT>::KW>::t pl,
-                                         typename Comp<Key<DT>::KW>::t pr) {
-    if (__any_sync(0xffffffffu, qs.cnt)) lq_flush<DT>(q, qs, sink, lo, pl, pr);
-    if (qs.pmax) lq_write<DT>(q.k[qs.cq ^ 1u], q.i[qs.cq ^ 1u], qs.pcnt, qs.pmax, qs.ra, qs.rb, sink, lo, pl, pr);
+                                         typename Comp<Key<DT>::KW>::t pr, const Bins& bins = Bins{}) {
+    if (__any_sync(0xffffffffu, qs.cnt)) lq_flush<DT>(q, qs, sink, lo, pl, pr, bins);
+    if (qs.pmax) lq_write<DT>(q.k[qs.cq ^ 1u], q.i[qs.cq ^ 1u], qs.pcnt, qs.pmax, qs.ra, qs.rb, sink, lo, pl, pr,
+                                 bins);
     qs.pmax = 0;
     __syncwarp();
 }
@@ -793,10 +825,11 @@ __device__ __forceinline__ void lq_drain(WarpQ<Key<DT>::KW>& q, LQState& qs, con
 // Each lane appends its own hits (bit q of `hit`: slot q; key_at(q) and
 // pos(q) for a lane-dependent q) to its part of the active buffer; a flush
 // first when some lane's part would overflow.  All 32 lanes call.
-template <int DT, class PosF, class KeyAt>
+template <int DT, class PosF, class KeyAt, class Bins = NoBins>
 __device__ __forceinline__ void lq_append(u32 hit, PosF pos, KeyAt key_at, typename Comp<Key<DT>::KW>::t lo,
                                           typename Comp<Key<DT>::KW>::t pl, typename Comp<Key<DT>::KW>::t pr,
-                                          const Sink<DT>& sink, WarpQ<Key<DT>::KW>& q, LQState& qs) {
+                                          const Sink<DT>& sink, WarpQ<Key<DT>::KW>& q, LQState& qs,
+                                          const Bins& bins = Bins{}) {
     constexpr u32 PER_LANE = LQ<Key<DT>::KW>::PER_LANE, CH = LQ<Key<DT>::KW>::CH;
     if (!__any_sync(0xffffffffu, hit)) return;
     const u32 lane = lane_id();
@@ -806,7 +839,7 @@ __device__ __forceinline__ void lq_append(u32 hit, PosF pos, KeyAt key_at, typen
 #pragma unroll 1
         for (u32 h = 0; h < 16 / CH; ++h) {
             u32 m = (hit >> (CH * h)) & ((1u << CH) - 1u);
-            if (__any_sync(0xffffffffu, qs.cnt + (u32)__popc(m) > PER_LANE)) lq_flush<DT>(q, qs, sink, lo, pl, pr);
+            if (__any_sync(0xffffffffu, qs.cnt + (u32)__popc(m) > PER_LANE)) lq_flush<DT>(q, qs, sink, lo, pl, pr, bins);
             while (m) {
                 const u32 sq = CH * h + (u32)(__ffs(m) - 1);
                 m &= m - 1;
@@ -840,10 +873,10 @@ template <class T> __device__ __forceinline__ T pick16(const T (&r)[16], u32 q) 
 }
 
 // Register path in sparse mode.
-template <int NT, int DT, class Src>
+template <int NT, int DT, class Src, class Bins>
 __device__ void pass_tiles_sparse(const Src& src, u64 tile0, u64 tile_step, typename Comp<Src::KW>::t lo,
                                   typename Comp<Src::KW>::t pl, typename Comp<Src::KW>::t pr, const Sink<DT>& sink,
-                                  WarpQ<Key<DT>::KW>& q) {
+                                  WarpQ<Key<DT>::KW>& q, const Bins& bins) {
     typedef typename Src::key_t key_t;
     constexpr u64 TILE = (u64)NT * 16;
     typedef Comp<Src::KW> C;
@@ -861,17 +894,17 @@ __device__ void pass_tiles_sparse(const Src& src, u64 tile0, u64 tile_step, type
         u32 hit = 0;
 #pragma unroll
         for (int s = 0; s < 16; ++s) hit |= (u32)(C::make(kk[s], pos(s)) <= pr) << s;
-        lq_append<DT>(hit & valid, pos, [&](u32 sq) { return pick16(kk, sq); }, lo, pl, pr, sink, q, qs);
+        lq_append<DT>(hit & valid, pos, [&](u32 sq) { return pick16(kk, sq); }, lo, pl, pr, sink, q, qs, bins);
     }
-    lq_drain<DT>(q, qs, sink, lo, pl, pr);
+    lq_drain<DT>(q, qs, sink, lo, pl, pr, bins);
 }
 
 // Register path: every thread loads its 16 elements of each tile itself.
-template <int NT, bool HAS_A, bool EXACT, int DT, class Src>
+template <int NT, bool HAS_A, bool EXACT, int DT, class Src, class Bins = NoBins>
 __device__ void pass_tiles(const Src& src, u64 tile0, u64 tile_step,
                            typename Comp<Src::KW>::t lo, typename Comp<Src::KW>::t pl,
                            typename Comp<Src::KW>::t pr, const Sink<DT>& sink,
-                           PassSmem<NT>& sm) {
+                           PassSmem<NT>& sm, const Bins& bins = Bins{}) {
     typedef typename Src::key_t key_t;
     constexpr u64 TILE = (u64)NT * 16;
     const u64 ntiles = (src.extent() + TILE - 1) / TILE;
@@ -884,7 +917,7 @@ __device__ void pass_tiles(const Src& src, u64 tile0, u64 tile_step,
             if constexpr (Src::IMPLICIT_IDX) return src.template idx_of<NT>(tb, s);
             else return ii[s];
         };
-        classify_emit<NT, HAS_A, EXACT, SyncBlock>(kk, pos, valid, lo, pl, pr, sink, sm);
+        classify_emit<NT, HAS_A, EXACT, SyncBlock>(kk, pos, valid, lo, pl, pr, sink, sm, bins);
     }
 }
 

@@ -1,19 +1,22 @@
 // select_impl.cuh — topk_select: selection of the k smallest of n unsorted keys
 // (paper, Section 2, Algorithm "select"; Section 4.1, Theorem "selectFR").
 //
-// Launch sequence of one call (all on the caller's stream, no host round
-// trip), per recursion level:
-//   k_sample (grid)     per-partition draws of the current window -> sample
-//                       array (draw j at slot j)
-//   k_pivots (1 block)  pivots = sample elements of ranks k|S|/n -/+ Delta:
-//                       the sample into shared memory, one histogram over
-//                       its range, the two rank bins ranked exactly
-//   k_pass   (grid)     one read of the source: a -> output, b -> candidate
-//                       buffer; the last block takes the branch
-// then k_finish (1 block): remaining levels inside one block until at most T
-// candidates are left, selection of rank k among them, the rest of the output
-// and the rank-k pair.  The host predicts the number of grid levels; a level
-// whose state is already small returns at once.
+// Launch sequence of one call (all on the caller's stream, no host round trip):
+//   k_plan   (1 cluster) sample of the input; pivots = its elements of ranks
+//                        k|S|/n -/+ Delta
+//   first pass  (grid)   one read of the input: a -> output, b -> candidate
+//                        buffer, the candidates also counted over equal bins;
+//                        the last block takes the branch and, when more
+//                        candidates are left than the finish holds, arms a
+//                        second pass between the ends of rank k's bin
+//   k_pass   (grid)      that second pass, over the candidates (usually a few
+//                        thousand are left); returns at once when not armed
+//   k_finish (1 cluster) selection of rank k among what is left, the rest of
+//                        the output and the rank-k pair
+// Inputs of at most T keys take k_finish alone.
+// Each recursion level used to sample anew (k_sample, k_pivots: about 17 us) before
+// its pass, two or three times a call; the bins give the second level exact
+// counts for nothing and narrow by a factor of about 1000 instead of 30.
 // k = 1 (the base case of Algorithm "select", a global minimum) and k = n
 // (everything selected) take one reduction kernel instead.
 #pragma once
@@ -24,7 +27,7 @@
 #include <mutex>
 
 #include "internal.h"
-#include "select_block.cuh"
+#include "select_cluster.cuh"
 
 namespace topk {
 
@@ -36,27 +39,78 @@ __device__ __forceinline__ u64 atomic_read(u64* p) {
 }
 
 // The branch of Algorithm "select", taken by the last block of a pass once
-// every block's counts are in (block-done counter; nobody waits).  The calling
-// thread must be the block's thread 0, after the block's own atomics.
-__device__ __forceinline__ void pass_epilogue(const SelArgs& a) {
-    __threadfence();
-    const u32 prev = atomicAdd(a.pass_done, 1u);
-    if (prev == gridDim.x - 1) {
+// every block's counts are in (block-done counter; nobody waits), and, after a
+// first level that leaves more candidates than the finish holds, the pivots of a
+// second pass: the ends of the bin that holds rank k (exact counts, so that pass
+// cannot miss).  All NT threads call, after the block's own atomics.
+struct EpilogueSmem {
+    u32 last, arm, wsum[32];
+};
+template <int KW, int NT, class Sync, bool BINS>
+__device__ __forceinline__ void pass_epilogue(const SelArgs& a, EpilogueSmem& es) {
+    typedef typename Comp<KW>::t ct;
+    Sync::sync();
+    if (threadIdx.x == 0) {
         __threadfence();
-        SelState* g = a.st;
+        es.last = atomicAdd(a.pass_done, 1u) == gridDim.x - 1;
+    }
+    Sync::sync();
+    if (!es.last) return;
+    SelState* g = a.st;
+    if (threadIdx.x == 0) {
+        __threadfence();
         g->cnt_a = atomic_read(&g->cnt_a);
         g->cnt_b = atomic_read(&g->cnt_b);
         decide(*g);
         *a.pass_done = 0;
+        es.arm = a.bins && g->src != SRC_INPUT && g->m_src > a.list_max && g->phase == PH_RUN;
+    }
+    if constexpr (BINS) {
+        Sync::sync();
+        if (!es.arm) return;
+        constexpr u32 PER = HB_BINS / NT; // consecutive bins per thread
+        static_assert(HB_BINS % NT == 0, "bins per thread");
+        const u32 lane = lane_id(), warp = threadIdx.x >> 5;
+        u32 h[PER], t = 0;
+#pragma unroll
+        for (u32 q = 0; q < PER; ++q) {
+            h[q] = __ldcg(a.bins->h + threadIdx.x * PER + q);
+            t += h[q];
+        }
+        u32 incl = t;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const u32 y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= (u32)o) incl += y;
+        }
+        if (lane == 31) es.wsum[warp] = incl;
+        Sync::sync();
+        for (u32 w = 0; w < warp; ++w) incl += es.wsum[w];
+        const u32 r = (u32)(*(volatile u64*)&g->k_rem - 1), nb = (u32) * (volatile u64*)&g->m_src;
+        u32 run = incl - t;
+#pragma unroll
+        for (u32 q = 0; q < PER; ++q) {
+            if (h[q] && r >= run && r < run + h[q] && h[q] < nb) { // one thread at most
+                const u32 b = threadIdx.x * PER + q;
+                const u32 sh = a.bins->shift;
+                const ct base = Comp<KW>::from128(a.bins->base), lo = Comp<KW>::from128(g->lo), hi = Comp<KW>::from128(g->hi);
+                // the end bins also hold what lies beyond them
+                const ct l = unpacked_comp<KW>((ct)(base + ((ct)b << sh)), a.idx_bits);
+                const ct u = unpacked_comp<KW>((ct)(base + (((ct)b + 1) << sh) - 1), a.idx_bits);
+                g->pl = (u128)(b == 0 || l < lo ? lo : l);
+                g->pr = (u128)(b == HB_BINS - 1 || u > hi || u < l ? hi : u);
+                g->dst = g->src == SRC_CAND0 ? SRC_CAND1 : SRC_CAND0;
+                g->cnt_a = 0;
+                g->cnt_b = 0;
+                g->dense = run > nb / 16 ? 1u : 0u;
+                g->level += 1;
+                g->levels_grid += 1;
+                g->pending = 1;
+            }
+            run += h[q];
+        }
     }
 }
-
-// ---- pickPivots: the sample (k_sample, whole grid) and the pivots
-// (k_pivots, one block), defined with the sampling routines further down.
-constexpr int SMP_NT = 128;
-constexpr int SMP_DRAWS = 4;        // one Philox block per thread
-constexpr u32 SMP_MAX_SCALE = 4;    // extra draws for a narrowed window
-constexpr int PIV_NT = 1024;
 
 // ---- partition + reduction + branch (whole grid)
 
@@ -77,52 +131,68 @@ __device__ __forceinline__ Sink<DT> make_sink(const SelArgs& a, const SelState& 
     return sink;
 }
 
-// Register-path pass (later levels; a first level on misaligned input).
-template <int DT, bool INPUT_ONLY> __device__ void grid_pass(const SelArgs& a, const SelState& s) {
-    typedef Key<DT> K;
-    typedef typename K::key_t key_t;
-    constexpr int KW = K::KW;
+// The bins of the first level's candidates in a block's shared memory.
+template <int DT>
+__device__ __forceinline__ BinHist<Key<DT>::KW> make_bins(const SelArgs& a, u32* h) {
+    if (!a.bins) return BinHist<Key<DT>::KW>{nullptr, 0, 0, 0};
+    return BinHist<Key<DT>::KW>{h, Comp<Key<DT>::KW>::from128(a.bins->base), a.bins->shift, a.idx_bits};
+}
+// Adds a block's bins to the grid's (NT threads, after a barrier).
+template <int NT> __device__ __forceinline__ void add_bins(const SelArgs& a, const u32* h) {
+    if (!a.bins) return;
+    for (u32 i = threadIdx.x; i < HB_BINS; i += NT)
+        if (h[i]) atomicAdd(a.bins->h + i, h[i]);
+}
+
+// Register-path pass (the second level; a first level on misaligned input).
+template <int NT, int DT, class Src, class Bins>
+__device__ __forceinline__ void pass_any(const Src& src, bool dense, typename Comp<Src::KW>::t lo,
+                                         typename Comp<Src::KW>::t pl, typename Comp<Src::KW>::t pr,
+                                         const Sink<DT>& sink, PassSmem<NT>& ps, WarpQ<Src::KW>& q, const Bins& bins) {
+    typedef typename Comp<Src::KW>::t ct;
+    if (!dense) pass_tiles_sparse<NT, DT>(src, blockIdx.x, gridDim.x, lo, pl, pr, sink, q, bins);
+    else if (lo != (ct)0) pass_tiles<NT, true, true, DT>(src, blockIdx.x, gridDim.x, lo, pl, pr, sink, ps, bins);
+    else pass_tiles<NT, true, false, DT>(src, blockIdx.x, gridDim.x, lo, pl, pr, sink, ps, bins);
+}
+
+// First level on misaligned input.
+template <int DT> __global__ void __launch_bounds__(PASS_NT) k_pass_first(SelArgs a) {
+    constexpr int KW = Key<DT>::KW;
     typedef Comp<KW> C;
-    typedef typename C::t ct;
     __shared__ PassSmem<PASS_NT> ps;
     __shared__ WarpQ<KW> wq[PASS_NT / 32];
-    const Sink<DT> sink = make_sink<DT>(a, s);
-    const ct lo = C::from128(s.lo), pl = C::from128(s.pl), pr = C::from128(s.pr);
-    const bool dense = s.dense != 0, exact = lo != (ct)0, has_a = pl > lo;
-    WarpQ<KW>& q = wq[threadIdx.x >> 5];
-    if (INPUT_ONLY || s.src == SRC_INPUT) {
-        const InputSrc<DT> src = InputSrc<DT>::make(a.keys, s.m_src);
-        if (!dense) pass_tiles_sparse<PASS_NT, DT>(src, blockIdx.x, gridDim.x, lo, pl, pr, sink, q);
-        else if (exact) pass_tiles<PASS_NT, true, true, DT>(src, blockIdx.x, gridDim.x, lo, pl, pr, sink, ps);
-        else if (has_a) pass_tiles<PASS_NT, true, false, DT>(src, blockIdx.x, gridDim.x, lo, pl, pr, sink, ps);
-        else pass_tiles<PASS_NT, false, false, DT>(src, blockIdx.x, gridDim.x, lo, pl, pr, sink, ps);
-    } else if constexpr (!INPUT_ONLY) {
-        const CandSrc<KW> src{static_cast<const key_t*>(a.cand_key[s.src - 1]), a.cand_idx[s.src - 1], s.m_src};
-        if (!dense) pass_tiles_sparse<PASS_NT, DT>(src, blockIdx.x, gridDim.x, lo, pl, pr, sink, q);
-        else if (exact) pass_tiles<PASS_NT, true, true, DT>(src, blockIdx.x, gridDim.x, lo, pl, pr, sink, ps);
-        else if (has_a) pass_tiles<PASS_NT, true, false, DT>(src, blockIdx.x, gridDim.x, lo, pl, pr, sink, ps);
-        else pass_tiles<PASS_NT, false, false, DT>(src, blockIdx.x, gridDim.x, lo, pl, pr, sink, ps);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) pass_epilogue(a);
-}
-
-// First level: the source is always the input, so this variant carries no
-// candidate-source code (fewer registers on the pass that reads all n keys).
-template <int DT> __global__ void __launch_bounds__(PASS_NT) k_pass_first(SelArgs a) {
+    __shared__ u32 hist[HB_BINS];
+    __shared__ EpilogueSmem es;
+    for (u32 i = threadIdx.x; i < HB_BINS; i += PASS_NT) hist[i] = 0;
     grid_dep_wait();
-    grid_dep_release();
     const SelState s = *a.st;
     if (s.phase != PH_RUN || !s.pending || s.src != SRC_INPUT) return;
-    grid_pass<DT, true>(a, s);
+    __syncthreads();
+    const BinHist<KW> bins = make_bins<DT>(a, hist);
+    pass_any<PASS_NT, DT>(InputSrc<DT>::make(a.keys, s.m_src), s.dense != 0, C::from128(s.lo), C::from128(s.pl),
+                          C::from128(s.pr), make_sink<DT>(a, s), ps, wq[threadIdx.x >> 5], bins);
+    grid_dep_release();
+    __syncthreads();
+    add_bins<PASS_NT>(a, hist);
+    pass_epilogue<KW, PASS_NT, SyncBlock, true>(a, es);
 }
 
+// Second level, over the candidates of the first, when its last block armed it.
 template <int DT> __global__ void __launch_bounds__(PASS_NT) k_pass(SelArgs a) {
+    typedef Key<DT> K;
+    constexpr int KW = K::KW;
+    typedef Comp<KW> C;
+    __shared__ PassSmem<PASS_NT> ps;
+    __shared__ WarpQ<KW> wq[PASS_NT / 32];
+    __shared__ EpilogueSmem es;
     grid_dep_wait();
     grid_dep_release();
     const SelState s = *a.st;
-    if (s.phase != PH_RUN || !s.pending) return;
-    grid_pass<DT, false>(a, s);
+    if (s.phase != PH_RUN || !s.pending || s.src == SRC_INPUT) return;
+    const CandSrc<KW> src{static_cast<const typename K::key_t*>(a.cand_key[s.src - 1]), a.cand_idx[s.src - 1], s.m_src};
+    pass_any<PASS_NT, DT>(src, s.dense != 0, C::from128(s.lo), C::from128(s.pl), C::from128(s.pr), make_sink<DT>(a, s),
+                          ps, wq[threadIdx.x >> 5], NoBins{});
+    pass_epilogue<KW, PASS_NT, SyncBlock, false>(a, es);
 }
 
 // First level, 16-byte-aligned input: a producer warp streams full tiles
@@ -144,7 +214,7 @@ template <int DT, int MODE = PM_SPARSE> struct TmaCfg {
     static constexpr u32 W = sizeof(typename Key<DT>::raw_t);
     static constexpr u32 TILE = TMA_CONS * 16; // elements per stage
     static constexpr u32 BYTES = TILE * W;     // 8, 16 or 32 KiB
-    static constexpr u32 STAGES = DENSE ? (W == 2 ? 8 : W == 4 ? 4 : 3) : (W == 2 ? 8 : W == 4 ? 5 : 3);
+    static constexpr u32 STAGES = W == 2 ? 8 : W == 4 ? 4 : 3; // two blocks (dense: three) fit an SM
     static constexpr u32 SMEM = STAGES * BYTES;
     static constexpr int MIN_BLOCKS = DENSE ? (W == 8 ? 2 : 3) : 1;
 };
@@ -160,13 +230,111 @@ __device__ __forceinline__ void load_raw_stage(const unsigned char* stage, typen
     InputSrc<DT>::unpack_raw(v, rr);
 }
 
-// Sparse first level (few elements in a and b): the elements whose pair is
-// at most pr are appended to the warp's queue (select_core.cuh); a tile that
-// contains neither pivot's position finds them with one comparison of raw
-// key bits per element (tile_bounds), the rare other tile on the pair.
-template <int DT>
-__device__ void tma_consume_sparse(const SelArgs& a, const SelState& s, const unsigned char* stages, uint64_t* full,
-                                   uint64_t* empty, u64 my_n, u32* dead, WarpQ<Key<DT>::KW>& wq) {
+// A warp's buffer of elements on their way out of a first-level pass, packed:
+// a tile's hits take consecutive slots (one shared-memory atomic per lane that has
+// any), so a flush writes whole rows of 32.  One flush in about 30 tiles waits
+// for its reservation, which the other warps and the ring cover.  (Per-lane
+// queues, whose rows are as long as the fullest lane's, and which classified every
+// entry again, took 0.27 ms for the counting pass on 2^28 f32 keys at k = n / 2,
+// 0.33 ms with the bins kept; packed: 0.235 ms with the bins.)
+template <int KW> struct WarpBuf {
+    static constexpr u32 CAP = KW == 32 ? 512 : 256; // a tile's 512 hits, or half of them
+    typename Comp<KW>::key_t k[CAP];
+    u32 i[CAP];
+    u32 n;
+};
+
+// Writes a warp's `cnt` entries (all at most pr): those below pl to the output,
+// unless the buffer holds b elements only (ONLY_B), the rest to the
+// candidates and their bins.
+template <int DT, bool ONLY_B>
+__device__ __forceinline__ void wb_flush(WarpBuf<Key<DT>::KW>& w, u32 cnt, typename Comp<Key<DT>::KW>::t pl,
+                                         const Sink<DT>& sink, const BinHist<Key<DT>::KW>& bins) {
+    typedef Comp<Key<DT>::KW> C;
+    const u32 lane = lane_id(), below = lanemask_lt();
+    __syncwarp();
+    u32 ca = 0;
+    if constexpr (!ONLY_B) {
+        for (u32 j = lane; j < cnt; j += 32) ca += (u32)(C::make(w.k[j], w.i[j]) < pl);
+        ca = __reduce_add_sync(0xffffffffu, ca);
+    }
+    u64 ra = 0, rb = 0;
+    if (lane == 0) {
+        if (!ONLY_B && ca) ra = atomicAdd((unsigned long long*)sink.cnt_a, (unsigned long long)ca);
+        if (cnt > ca) rb = atomicAdd((unsigned long long*)sink.cnt_b, (unsigned long long)(cnt - ca));
+        w.n = 0;
+    }
+    if constexpr (!ONLY_B) ra = __shfl_sync(0xffffffffu, (unsigned long long)ra, 0);
+    rb = __shfl_sync(0xffffffffu, (unsigned long long)rb, 0);
+    for (u32 j0 = 0; j0 < cnt; j0 += 32) {
+        const u32 j = j0 + lane;
+        const bool in = j < cnt;
+        const auto kv = in ? w.k[j] : (typename C::key_t)0;
+        const u32 iv = in ? w.i[j] : 0u;
+        if constexpr (ONLY_B) {
+            if (in) {
+                sink.put_b(rb + j, kv, iv);
+                bins.add(kv, iv);
+            }
+        } else {
+            const bool isa = in && C::make(kv, iv) < pl;
+            const u32 bala = __ballot_sync(0xffffffffu, isa), balb = __ballot_sync(0xffffffffu, in && !isa);
+            if (isa) sink.put_a(ra + __popc(bala & below), kv, iv); // (writes nothing where cap_a = 0)
+            else if (in) {
+                sink.put_b(rb + __popc(balb & below), kv, iv);
+                bins.add(kv, iv);
+            }
+            ra += __popc(bala);
+            rb += __popc(balb);
+        }
+    }
+    __syncwarp();
+}
+
+// Appends the slots of `hit` (key_at(q), pos(q) for a lane-dependent q); `cnt` is
+// the number of entries, the same in every lane.  All 32 lanes call.
+template <int DT, bool ONLY_B, class PosF, class KeyAt>
+__device__ __forceinline__ void wb_append(WarpBuf<Key<DT>::KW>& w, u32& cnt, u32 hit, PosF pos, KeyAt key_at,
+                                          typename Comp<Key<DT>::KW>::t pl, const Sink<DT>& sink,
+                                          const BinHist<Key<DT>::KW>& bins) {
+    constexpr u32 CAP = WarpBuf<Key<DT>::KW>::CAP;
+    constexpr u32 PARTS = 512 / CAP; // slots taken at once: as many as always fit
+    if (!__any_sync(0xffffffffu, hit)) return;
+    const u32 all = hit;
+#pragma unroll 1
+    for (u32 h = 0; h < PARTS; ++h) {
+        u32 m = PARTS == 1 ? all : (all >> (h * (16 / PARTS)) << (h * (16 / PARTS))) & ((1u << ((h + 1) * (16 / PARTS))) - 1u);
+        const u32 mine = (u32)__popc(m);
+        const u32 total = __reduce_add_sync(0xffffffffu, mine);
+        if (cnt + total > CAP) {
+            wb_flush<DT, ONLY_B>(w, cnt, pl, sink, bins);
+            cnt = 0;
+        }
+        if (m) {
+            u32 slot = atomicAdd(&w.n, mine);
+            do {
+                const u32 q = (u32)(__ffs(m) - 1);
+                m &= m - 1;
+                w.k[slot] = key_at(q);
+                w.i[slot] = pos((int)q);
+                ++slot;
+            } while (m);
+        }
+        cnt += total;
+    }
+}
+
+// First level with few elements to write (sparse: a and b both; counting: b, a
+// being counted in registers and never written, for a call that wants the
+// rank-k pair alone).  A tile that holds neither pivot's position is tested
+// with one comparison of raw key bits per element and pivot (tile bounds), the
+// rare other tile on the pair; the few hits go through the warp's buffer.  No
+// block barrier.  On 2^28 f32 keys at k = n / 2 the counting pass takes 0.235
+// ms, against 0.47 ms for the pass that writes a.
+template <int DT, bool COUNT>
+__device__ void tma_consume_few(const SelArgs& a, const SelState& s, const unsigned char* stages, uint64_t* full,
+                                uint64_t* empty, u64 my_n, u32* dead, WarpBuf<Key<DT>::KW>& wb,
+                                const BinHist<Key<DT>::KW>& bins) {
     typedef Key<DT> K;
     typedef typename K::raw_t raw_t;
     typedef typename K::key_t key_t;
@@ -175,14 +343,15 @@ __device__ void tma_consume_sparse(const SelArgs& a, const SelState& s, const un
     typedef TmaCfg<DT> Cfg;
     constexpr u32 EPV = InputSrc<DT>::EPV;
     const Sink<DT> sink = make_sink<DT>(a, s);
-    const ct lo = C::from128(s.lo), pl = C::from128(s.pl), pr = C::from128(s.pr);
+    const ct pl = C::from128(s.pl), pr = C::from128(s.pr);
     const u32 lane = lane_id();
     const InputSrc<DT> isrc = InputSrc<DT>::make(a.keys, s.m_src); // head = 0: input is 16-byte aligned
-    LQState qs = LQState::make();
+    if (lane == 0) wb.n = 0;
+    __syncwarp();
     const TileBounds<DT> tbd = TileBounds<DT>::make(pl, pr);
+    u64 na = 0;
+    u32 cnt = 0, stg = 0, parity = 0;
     for (u64 i = 0; i < my_n; ++i) {
-        const u32 stg = (u32)(i % Cfg::STAGES);
-        const u32 parity = (u32)((i / Cfg::STAGES) & 1);
         bool ok = !*(volatile u32*)dead;
         if (ok && !mbar_wait_bounded(&full[stg], parity, WAIT_LIMIT_NS)) {
             ok = false;
@@ -195,82 +364,6 @@ __device__ void tma_consume_sparse(const SelArgs& a, const SelState& s, const un
         const u32 tb = (u32)((blockIdx.x + i * gridDim.x) * (u64)Cfg::TILE);
         const u32 ib = tb + threadIdx.x * EPV;
         auto pos = [&](int q) -> u32 { return ib + (u32)(q / (int)EPV) * (TMA_CONS * EPV) + (u32)(q % (int)EPV); };
-        raw_t rr[16];
-        u32 hit = 0;
-        if (ok) {
-            load_raw_stage<DT>(stages + (size_t)stg * Cfg::BYTES, rr);
-            RawBound<DT> ba, bb;
-            bool any_a, any_l;
-            if (tbd.get(tb, tb + Cfg::TILE - 1, ba, bb, any_a, any_l)) {
-                hit = tile_le_dispatch<DT>(rr, bb, any_l);
-            } else {
-#pragma unroll
-                for (int q = 0; q < 16; ++q) hit |= (u32)(C::make(K::fwd(rr[q]), pos(q)) <= pr) << q;
-            }
-        } else {
-#pragma unroll
-            for (int q = 0; q < 16; ++q) rr[q] = 0;
-        }
-        // the hits' keys come from the stage, which is released after them
-        const unsigned char* mine = stages + (size_t)stg * Cfg::BYTES + threadIdx.x * 16u;
-        lq_append<DT>(hit, pos, [&](u32 sq) {
-            return K::fwd(*reinterpret_cast<const raw_t*>(mine + (sq / EPV) * (TMA_CONS * 16u) + (sq % EPV) * sizeof(raw_t)));
-        }, lo, pl, pr, sink, wq, qs);
-        __syncwarp();
-        if (ok && lane == 0) mbar_arrive(&empty[stg]); // the stage may be refilled
-    }
-    // the ragged last tile, read directly by the block that owns it
-    const u64 nfull = s.m_src / Cfg::TILE;
-    if (s.m_src % Cfg::TILE != 0 && nfull % gridDim.x == blockIdx.x) {
-        key_t kk[16];
-        u32 ii[16];
-        const u64 tb = nfull * (u64)Cfg::TILE;
-        const u32 valid = isrc.template load16<TMA_CONS>(tb, kk, ii);
-        auto pos = [&](int q) -> u32 { return isrc.template idx_of<TMA_CONS>(tb, q); };
-        u32 tail_hit = 0;
-#pragma unroll
-        for (int q = 0; q < 16; ++q) tail_hit |= (u32)(C::make(kk[q], pos(q)) <= pr) << q;
-        lq_append<DT>(tail_hit & valid, pos, [&](u32 sq) { return pick16(kk, sq); }, lo, pl, pr, sink, wq, qs);
-    }
-    lq_drain<DT>(wq, qs, sink, lo, pl, pr);
-}
-
-// First level of a call that wants the rank-k pair alone, with many elements
-// in a: a is counted in registers and never written, only the few b elements
-// leave (through the warp queues).  Two comparisons of raw key bits per key and
-// no barrier or reservation for a, so the pass streams at memory speed, where
-// the emitting pass below is bound by its instructions and twice the bytes.
-// On 2^28 f32 keys at k = n / 2: 0.27 ms for the pass, against 0.47 ms for
-// the emitting one.
-template <int DT>
-__device__ void tma_consume_count(const SelArgs& a, const SelState& s, const unsigned char* stages, uint64_t* full,
-                                  uint64_t* empty, u64 my_n, u32* dead, WarpQ<Key<DT>::KW>& wq) {
-    typedef Key<DT> K;
-    typedef typename K::raw_t raw_t;
-    typedef typename K::key_t key_t;
-    typedef Comp<K::KW> C;
-    typedef typename C::t ct;
-    typedef TmaCfg<DT> Cfg;
-    constexpr u32 EPV = InputSrc<DT>::EPV;
-    const Sink<DT> sink = make_sink<DT>(a, s);
-    const ct pl = C::from128(s.pl), pr = C::from128(s.pr);
-    const u32 lane = lane_id();
-    const InputSrc<DT> isrc = InputSrc<DT>::make(a.keys, s.m_src); // head = 0: input is 16-byte aligned
-    LQState qs = LQState::make();
-    const TileBounds<DT> tbd = TileBounds<DT>::make(pl, pr);
-    u64 na = 0;
-    u32 stg = 0, parity = 0;
-    for (u64 i = 0; i < my_n; ++i) {
-        bool ok = !*(volatile u32*)dead;
-        if (ok && !mbar_wait_bounded(&full[stg], parity, WAIT_LIMIT_NS)) {
-            ok = false;
-            *(volatile u32*)dead = 1;
-            if (lane == 0) latch(a.err, ST_ETIMEOUT);
-        }
-        ok = __all_sync(0xffffffffu, ok);
-        const u32 tb = (u32)((blockIdx.x + i * gridDim.x) * (u64)Cfg::TILE);
-        const u32 ib = tb + threadIdx.x * EPV;
-        auto pos = [&](int q) -> u32 { return ib + (u32)(q / (int)EPV) * (TMA_CONS * EPV) + (u32)(q % (int)EPV); };
         u32 ma = 0, le = 0;
         if (ok) {
             raw_t rr[16];
@@ -278,21 +371,23 @@ __device__ void tma_consume_count(const SelArgs& a, const SelState& s, const uns
             RawBound<DT> ba, bb;
             bool any_a, any_l;
             if (tbd.get(tb, tb + Cfg::TILE - 1, ba, bb, any_a, any_l)) {
-                tile_masks_dispatch<DT>(rr, ba, bb, any_a, any_l, ma, le);
+                if constexpr (COUNT) tile_masks_dispatch<DT>(rr, ba, bb, any_a, any_l, ma, le);
+                else le = tile_le_dispatch<DT>(rr, bb, any_l);
             } else {
 #pragma unroll
                 for (int q = 0; q < 16; ++q) {
                     const ct c = C::make(K::fwd(rr[q]), pos(q));
-                    ma |= (u32)(c < pl) << q;
+                    if (COUNT) ma |= (u32)(c < pl) << q;
                     le |= (u32)(c <= pr) << q;
                 }
             }
         }
-        na += (u32)__popc(ma);
+        if (COUNT) na += (u32)__popc(ma);
+        // the hits' keys come from the stage, which is released after them
         const unsigned char* mine = stages + (size_t)stg * Cfg::BYTES + threadIdx.x * 16u;
-        lq_append<DT>(le & ~ma, pos, [&](u32 sq) {
+        wb_append<DT, COUNT>(wb, cnt, le & ~ma, pos, [&](u32 sq) {
             return K::fwd(*reinterpret_cast<const raw_t*>(mine + (sq / EPV) * (TMA_CONS * 16u) + (sq % EPV) * sizeof(raw_t)));
-        }, (ct)0, pl, pr, sink, wq, qs);
+        }, pl, sink, bins);
         __syncwarp();
         if (ok && lane == 0) mbar_arrive(&empty[stg]); // the stage may be refilled
         if (++stg == Cfg::STAGES) {
@@ -312,17 +407,19 @@ __device__ void tma_consume_count(const SelArgs& a, const SelState& s, const uns
 #pragma unroll
         for (int q = 0; q < 16; ++q) {
             const ct c = C::make(kk[q], pos(q));
-            ma |= (u32)(c < pl) << q;
+            if (COUNT) ma |= (u32)(c < pl) << q;
             le |= (u32)(c <= pr) << q;
         }
         ma &= valid;
         na += (u32)__popc(ma);
-        lq_append<DT>(le & valid & ~ma, pos, [&](u32 sq) { return pick16(kk, sq); }, (ct)0, pl, pr, sink, wq, qs);
+        wb_append<DT, COUNT>(wb, cnt, le & valid & ~ma, pos, [&](u32 sq) { return pick16(kk, sq); }, pl, sink, bins);
     }
-    lq_drain<DT>(wq, qs, sink, (ct)0, pl, pr);
+    if (cnt) wb_flush<DT, COUNT>(wb, cnt, pl, sink, bins);
+    if constexpr (COUNT) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) na += __shfl_xor_sync(0xffffffffu, (unsigned long long)na, o);
-    if (lane == 0 && na) atomicAdd((unsigned long long*)sink.cnt_a, (unsigned long long)na);
+        for (int o = 16; o > 0; o >>= 1) na += __shfl_xor_sync(0xffffffffu, (unsigned long long)na, o);
+        if (lane == 0 && na) atomicAdd((unsigned long long*)sink.cnt_a, (unsigned long long)na);
+    }
 }
 
 // Dense first level (many elements in a; the window starts at the smallest
@@ -349,7 +446,8 @@ struct DenseSmem {
 
 template <int DT>
 __device__ void tma_consume_dense(const SelArgs& a, const SelState& s, const unsigned char* stages, uint64_t* full,
-                                  uint64_t* empty, u64 my_n, u32* dead, DenseSmem& ds, PassSmem<TMA_CONS>& ps) {
+                                  uint64_t* empty, u64 my_n, u32* dead, DenseSmem& ds, PassSmem<TMA_CONS>& ps,
+                                  const BinHist<Key<DT>::KW>& bins) {
     typedef Key<DT> K;
     typedef typename K::raw_t raw_t;
     typedef typename K::key_t key_t;
@@ -498,7 +596,10 @@ __device__ void tma_consume_dense(const SelArgs& a, const SelState& s, const uns
                 while (m) {
                     const u32 q = (u32)(__ffs(m) - 1);
                     m &= m - 1;
-                    sink.put_b(xb++, K::fwd(elem(q)), ib_prev + (q / EPV) * STRIDE + q % EPV);
+                    const key_t kb = K::fwd(elem(q));
+                    const u32 ibq = ib_prev + (q / EPV) * STRIDE + q % EPV;
+                    sink.put_b(xb++, kb, ibq);
+                    bins.add(kb, ibq);
                 }
             }
             __syncwarp();
@@ -518,7 +619,7 @@ __device__ void tma_consume_dense(const SelArgs& a, const SelState& s, const uns
         const u64 tb = nfull * (u64)Cfg::TILE;
         const u32 valid = isrc.template load16<TMA_CONS>(tb, kk, ii);
         auto pos = [&](int q) -> u32 { return isrc.template idx_of<TMA_CONS>(tb, q); };
-        classify_emit<TMA_CONS, true, false, Sync>(kk, pos, valid, (ct)0, pl, pr, sink, ps);
+        classify_emit<TMA_CONS, true, false, Sync>(kk, pos, valid, (ct)0, pl, pr, sink, ps, bins);
     }
 }
 
@@ -532,9 +633,12 @@ __global__ void __launch_bounds__(TMA_NT, (TmaCfg<DT, MODE>::MIN_BLOCKS)) k_pass
     __shared__ __align__(8) uint64_t full[Cfg::STAGES];
     __shared__ __align__(8) uint64_t empty[Cfg::STAGES];
     __shared__ PassSmem<TMA_CONS> ps;
-    __shared__ WarpQ<KW> wq[DENSE ? 1 : TMA_CONS / 32];
+    __shared__ __align__(16) unsigned char wb_raw[DENSE ? 16 : sizeof(WarpBuf<KW>) * (TMA_CONS / 32)];
     __shared__ DenseSmem ds;
+    __shared__ u32 hist[HB_BINS];
+    __shared__ EpilogueSmem es;
     __shared__ u32 dead;
+    for (u32 i = threadIdx.x; i < HB_BINS; i += TMA_NT) hist[i] = 0;
     grid_dep_wait();
     const SelState s = *a.st;
     if (s.phase != PH_RUN || !s.pending || s.src != SRC_INPUT || (s.dense != 0) != (MODE != PM_SPARSE)) {
@@ -547,7 +651,6 @@ __global__ void __launch_bounds__(TMA_NT, (TmaCfg<DT, MODE>::MIN_BLOCKS)) k_pass
         if (threadIdx.x == 0) latch(a.err, ST_EINTERNAL);
         return;
     }
-    // the working variant keeps the next kernel's blocks off its SMs until it ends
     if (threadIdx.x == 0) {
         for (u32 i = 0; i < Cfg::STAGES; ++i) {
             mbar_init(&full[i], 1);
@@ -583,294 +686,14 @@ __global__ void __launch_bounds__(TMA_NT, (TmaCfg<DT, MODE>::MIN_BLOCKS)) k_pass
         }
         return;
     }
-    WarpQ<KW>& q = wq[DENSE ? 0 : threadIdx.x >> 5];
-    if constexpr (MODE == PM_SPARSE) tma_consume_sparse<DT>(a, s, stages, full, empty, my_n, &dead, q);
-    else if constexpr (MODE == PM_COUNT) tma_consume_count<DT>(a, s, stages, full, empty, my_n, &dead, q);
-    else tma_consume_dense<DT>(a, s, stages, full, empty, my_n, &dead, ds, ps);
+    const BinHist<KW> bins = make_bins<DT>(a, hist);
+    WarpBuf<KW>* wb = reinterpret_cast<WarpBuf<KW>*>(wb_raw) + (DENSE ? 0 : threadIdx.x >> 5);
+    if constexpr (!DENSE) tma_consume_few<DT, MODE == PM_COUNT>(a, s, stages, full, empty, my_n, &dead, *wb, bins);
+    else tma_consume_dense<DT>(a, s, stages, full, empty, my_n, &dead, ds, ps, bins);
+    grid_dep_release(); // this block's stream has ended: the next kernel may start taking its place
     SyncNamed<1, TMA_CONS>::sync();
-    if (threadIdx.x == 0) pass_epilogue(a);
-}
-
-// Number of draws of a level: the sample size, more for a narrowed window
-// (proportionally, at most SMP_MAX_SCALE times), so that about as many land
-// inside it.
-__device__ __forceinline__ u32 level_draws(const SelArgs& a, const SelState& s) {
-    u32 draws = a.sample;
-    if (s.m_win < s.m_src) {
-        u64 ratio = s.m_src / (s.m_win ? s.m_win : 1);
-        ratio = ratio < 1 ? 1 : ratio > SMP_MAX_SCALE ? SMP_MAX_SCALE : ratio;
-        draws = (u32)((u64)draws * ratio);
-    }
-    return draws;
-}
-
-// Slots of the sample array a level fills: every draw when they all fit
-// (draw j at slot j), else the draws inside the window (appended, up to the
-// capacity).  `count` is the append counter.
-__device__ __forceinline__ u32 sample_stored(const SelArgs& a, u32 draws, const u32* count) {
-    if (draws <= a.samp_cap) return draws;
-    const u32 c = *(const volatile u32*)count;
-    return c < a.samp_cap ? c : a.samp_cap;
-}
-
-// The sample of one level, drawn by a grid of NT-thread blocks: draw j falls
-// in partition j mod p at a position uniform in it (Philox4x32-10 of counter
-// (4 floor(j / 4), level, salt, 0), word j mod 4).  When the draws fit the
-// sample array, draw j is stored at slot j (a draw outside the window as the
-// all-ones composite, which no element has); otherwise the draws inside the
-// window are appended (one reservation per warp on `count`).  The four draws
-// of one Philox block go to one thread; consecutive blocks of draws go to
-// consecutive thread blocks.
-template <int DT, int NT>
-__device__ void sample_draws(const SelArgs& a, const SelState& s, typename Comp<Key<DT>::KW>::t lo,
-                             typename Comp<Key<DT>::KW>::t hi, u32 draws, u32* count) {
-    typedef Key<DT> K;
-    typedef typename K::key_t key_t;
-    constexpr int KW = K::KW;
-    typedef Comp<KW> C;
-    typedef typename C::t ct;
-    const bool direct = draws <= a.samp_cap;
-    const u32 m = (u32)s.m_src; // sources hold fewer than 2^32 elements
-    const u32 p = a.parts < m ? a.parts : m;
-    const u32 len = m / p, rem = m - len * p;
-    const InputSrc<DT> isrc = InputSrc<DT>::make(a.keys, m);
-    const CandSrc<KW> csrc{static_cast<const key_t*>(a.cand_key[s.src == SRC_CAND1 ? 1 : 0]),
-                           a.cand_idx[s.src == SRC_CAND1 ? 1 : 0], m};
-    ct* samp = static_cast<ct*>(a.samp);
-    const u32 blocks4 = (draws + 3) / 4; // Philox blocks
-    // Philox block b = (round * NT + t) * gridDim.x + blockIdx.x for thread t
-    const u32 rounds = (blocks4 + gridDim.x * NT - 1) / (gridDim.x * NT);
-    for (u32 rd = 0; rd < rounds; ++rd) {
-        const u32 b = (rd * NT + threadIdx.x) * gridDim.x + blockIdx.x;
-        // warps whose blocks of draws all lie beyond the last stop here
-        const u32 warp_b0 = (rd * NT + (threadIdx.x & ~31u)) * gridDim.x + blockIdx.x;
-        if (warp_b0 >= blocks4) break;
-        ct c[4];
-        u32 keepm = 0;
-        const u32 j0 = b * 4;
-        if (b < blocks4) {
-            const Philox4 r = philox4x32_10(j0, s.level, 0x53414D50u, 0, (u32)a.seed, (u32)(a.seed >> 32));
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const u32 j = j0 + q;
-                const u32 part = j % p;
-                const u32 plo = part * len + (part < rem ? part : rem);
-                const u32 psz = len + (part < rem ? 1 : 0);
-                const u32 pos = plo + (u32)(((u64)r.v[q] * psz) >> 32);
-                key_t kq = 0;
-                u32 x = 0;
-                if (j < draws) {
-                    if (s.src == SRC_INPUT) isrc.at(pos, kq, x);
-                    else csrc.at(pos, kq, x);
-                }
-                c[q] = C::make(kq, x);
-                keepm |= (u32)(j < draws && c[q] >= lo && c[q] <= hi) << q;
-            }
-        }
-        if (direct) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (b < blocks4 && j0 + q < draws) samp[j0 + q] = ((keepm >> q) & 1u) ? c[q] : ~(ct)0;
-        } else {
-            u32 slot = warp_reserve((u32)__popc(keepm), count);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                if ((keepm >> q) & 1u) {
-                    if (slot < a.samp_cap) samp[slot] = c[q];
-                    ++slot;
-                }
-            }
-        }
-    }
-}
-
-// Pivots from the sample (one block of NT threads): the sample array
-// (`stored` slots) into shared memory `buf` by one bulk copy (completion on
-// the block's mbarrier `mb`, phase `mphase`), the number `kept` of draws in
-// the window and their smallest and largest composite; then the sample
-// elements of ranks k|S|/n -/+ Delta (pivot_ranks), selected with a histogram
-// over [smallest, largest].  Returns kept; pl / pr stay as given when a rank
-// falls outside the sample; *jl_out receives the lower rank.  `ok` turns
-// false if the copy did not complete in time.
-template <int DT, int NT>
-__device__ u32 sample_pivots(const SelArgs& a, const SelState& s, u32 stored, typename Comp<Key<DT>::KW>::t lo,
-                             typename Comp<Key<DT>::KW>::t hi, typename Comp<Key<DT>::KW>::t* buf,
-                             HistSelSmem<Key<DT>::KW>& hs, uint64_t* mb, u32& mphase, bool& ok,
-                             typename Comp<Key<DT>::KW>::t& pl, typename Comp<Key<DT>::KW>::t& pr,
-                             long long* jl_out) {
-    constexpr int KW = Key<DT>::KW;
-    typedef Comp<KW> C;
-    typedef typename C::t ct;
-    __shared__ ct s_mn[NT / 32], s_mx[NT / 32];
-    __shared__ u32 s_cnt[NT / 32];
-    __shared__ long long s_jl, s_jr;
-    __shared__ u32 s_kept;
-    const u32 tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
-    // the sample array holds a whole number of 16-byte words and starts on
-    // a 16-byte boundary, as does the shared copy
-    const u32 bytes = (u32)((stored * sizeof(ct) + 15) & ~(size_t)15);
-    __syncthreads(); // earlier readers of the shared sample are done
-    if (tid == 0 && bytes > 0) {
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        mbar_arrive_expect_tx(mb, bytes);
-        bulk_g2s(buf, a.samp, bytes, mb);
-    }
-    if (bytes > 0) {
-        if (!mbar_wait_bounded(mb, mphase, WAIT_LIMIT_NS)) {
-            ok = false;                                          // reported, and once more
-            (void)mbar_wait_bounded(mb, mphase, WAIT_LIMIT_NS); // for the copy in flight
-        }
-        mphase ^= 1u;
-    }
-    if (__syncthreads_or(ok ? 0 : 1)) ok = false; // the same answer in every thread
-    ct mn = ~(ct)0, mx = 0;
-    u32 cnt = 0;
-    for (u32 i = tid; i < stored; i += NT) {
-        const ct c = buf[i];
-        // (a window's upper end may be the all-ones composite itself, so the
-        // stand-in for a draw outside it is excluded by value)
-        const bool in = c != ~(ct)0 && c >= lo && c <= hi;
-        cnt += (u32)in;
-        if (in && c < mn) mn = c;
-        if (in && c > mx) mx = c;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const ct omn = shfl_comp(mn, lane ^ (u32)o), omx = shfl_comp(mx, lane ^ (u32)o);
-        mn = omn < mn ? omn : mn;
-        mx = omx > mx ? omx : mx;
-        cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-    }
-    if (lane == 0) {
-        s_mn[warp] = mn;
-        s_mx[warp] = mx;
-        s_cnt[warp] = cnt;
-    }
-    __syncthreads();
-    if (tid == 0) {
-        ct a_mn = s_mn[0], a_mx = s_mx[0];
-        u32 a_cnt = s_cnt[0];
-        for (u32 w = 1; w < NT / 32; ++w) {
-            a_mn = s_mn[w] < a_mn ? s_mn[w] : a_mn;
-            a_mx = s_mx[w] > a_mx ? s_mx[w] : a_mx;
-            a_cnt += s_cnt[w];
-        }
-        long long jl = -1, jr = 0;
-        if (a_cnt > 0) pivot_ranks(a_cnt, s.m_win, s.k_rem, a.z, (a.flags & TOPK_FLAG_RAW_DELTA) != 0, jl, jr);
-        s_jl = jl;
-        s_jr = jr;
-        s_kept = a_cnt;
-        s_mn[0] = a_mn;
-        s_mx[0] = a_mx;
-    }
-    __syncthreads();
-    const u32 kept = s_kept;
-    const long long jl = s_jl, jr = s_jr, top = (long long)kept - 1;
-    if (jl_out) *jl_out = jl;
-    if (kept > 0 && ok) {
-        ct x0, x1;
-        block_select_two<KW, NT>(buf, stored, s_mn[0], s_mx[0], (u32)(jl < 0 ? 0 : jl > top ? top : jl),
-                                 (u32)(jr < 0 ? 0 : jr > top ? top : jr), hs, x0, x1);
-        if (jl >= 0) pl = x0;
-        if (jr <= top) pr = x1;
-    }
-    return kept;
-}
-
-// ---- pickPivots, part 1 (whole grid): the level's draws into the sample
-// array (sample_draws).
-template <int DT> __global__ void __launch_bounds__(SMP_NT) k_sample(SelArgs a, int first) {
-    grid_dep_wait();
-    grid_dep_release();
-    typedef Comp<Key<DT>::KW> C;
-    const SelState s = first ? initial_state<DT>(a) : *a.st;
-    if (s.phase != PH_RUN || s.m_src <= a.grid_G || s.m_win <= a.finish_T) return;
-    sample_draws<DT, SMP_NT>(a, s, C::from128(s.lo), C::from128(s.hi), level_draws(a, s), a.samp_count);
-}
-
-// ---- pickPivots, part 2 (one block): the pivots from the sample
-// (sample_pivots), then the next pass armed; the sample count is left at zero
-// for the next level.  A window of at most T elements is collected whole.
-template <int KW> struct PivotSmem {
-    typedef typename Comp<KW>::t ct;
-    ct buf[Lim<KW>::ELEMS];
-    HistSelSmem<KW> hs;
-};
-
-template <int DT> __global__ void __launch_bounds__(PIV_NT) k_pivots(SelArgs a, int first) {
-    grid_dep_wait();
-    grid_dep_release();
-    constexpr int KW = Key<DT>::KW;
-    typedef Comp<KW> C;
-    typedef typename C::t ct;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    auto& sm = *reinterpret_cast<PivotSmem<KW>*>(smem_raw);
-    __shared__ __align__(8) uint64_t mb; // completion of the sample's bulk copy
-    __shared__ u32 s_go;
-    SelState* g = a.st;
-    const u32 tid = threadIdx.x;
-    const SelState s = first ? initial_state<DT>(a) : *g;
-    if (tid == 0) {
-        if (first) *g = s;
-        u32 go = s.phase == PH_RUN;
-        if (go && s.m_src <= a.grid_G) {
-            g->phase = PH_FINISH;
-            go = 0;
-        }
-        s_go = go;
-        mbar_init(&mb, 1);
-        mbar_fence_init();
-    }
-    __syncthreads();
-    if (!s_go) return;
-    const ct lo = C::from128(s.lo), hi = C::from128(s.hi);
-    ct pl = lo, pr = hi; // "collect": every window element becomes a candidate
-    u32 kept = 0, mphase = 0;
-    long long jl = -1;
-    bool ok = true;
-    if (s.m_win > a.finish_T) {
-        const u32 stored = sample_stored(a, level_draws(a, s), a.samp_count);
-        kept = sample_pivots<DT, PIV_NT>(a, s, stored, lo, hi, sm.buf, sm.hs, &mb, mphase, ok, pl, pr, &jl);
-    }
-    if (tid == 0) {
-        if (!ok) {
-            latch(a.err, ST_ETIMEOUT);
-            g->phase = PH_ERROR;
-        }
-        g->pl = (u128)pl;
-        g->pr = (u128)pr;
-        g->dst = s.src == SRC_CAND0 ? SRC_CAND1 : SRC_CAND0;
-        g->cnt_a = 0;
-        g->cnt_b = 0;
-        g->pending = 1;
-        g->level = s.level + 1;
-        g->levels_grid++;
-        if (s.level == 0) g->sample_kept = kept;
-        // many a-elements expected: the pass compacts with block scans (on
-        // the first level the host has chosen, by the same rule, the one
-        // variant it launches)
-        g->dense = (s.level == 0 && a.first_dense >= 0)
-                       ? (u32)a.first_dense
-                       : (jl >= 0 && kept > 0 && (double)(jl + 1) > (double)kept / 16.0) ? 1u : 0u;
-        *a.samp_count = 0;
-    }
-}
-
-// Remaining levels in one block, then the exact finish.
-template <int DT> __global__ void __launch_bounds__(BLK_NT) k_finish(SelArgs a, int first) {
-    grid_dep_wait();
-    grid_dep_release();
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    auto& sm = *reinterpret_cast<BlockSmem<Key<DT>::KW>*>(smem_raw);
-    SelState* g = a.st;
-    if (threadIdx.x == 0) {
-        if (first) init_state<DT>(g, a);
-        if (g->phase == PH_RUN) g->phase = PH_FINISH;
-        sm.flag = g->phase == PH_FINISH;
-    }
-    __syncthreads();
-    if (!sm.flag) return;
-    block_levels_and_finish<DT, true, true>(a, sm);
+    add_bins<TMA_CONS>(a, hist);
+    pass_epilogue<KW, TMA_CONS, SyncNamed<1, TMA_CONS>, true>(a, es);
 }
 
 // k = 1: the minimum pair (base case of Algorithm "select");
@@ -975,7 +798,7 @@ __global__ void __launch_bounds__(EXT_NT) k_extreme(SelArgs a, int want_max, u32
 // ----------------------------------------------------------- host side
 
 struct Tuning {
-    u32 sample, parts, T, G;
+    u32 sample, parts, T;
     float z;
     u32 flags;
     u64 seed;
@@ -989,7 +812,6 @@ template <int KW> static Tuning make_tuning(const topk_params* prm, int sms) {
     tu.sample = p.sample_size ? std::min<u32>(std::max<u32>(p.sample_size, 64), ELEMS) : ELEMS;
     tu.parts = p.partitions ? p.partitions : (u32)sms;
     tu.T = p.finish_threshold ? std::min<u32>(std::max<u32>(p.finish_threshold, 64), ELEMS) : ELEMS;
-    tu.G = tu.T; // grid levels run until the one-block finish can take over
     tu.z = p.delta_factor > 0.f ? p.delta_factor : 4.0f;
     tu.flags = p.flags;
     tu.seed = p.seed ? p.seed : 0x243F6A8885A308D3ull;
@@ -1010,17 +832,17 @@ static SelArgs make_args(const void* keys, u64 n, u64 k, void* out_keys, u32* ou
     a.parts = tu.parts;
     a.sample = tu.sample;
     a.finish_T = tu.T;
-    a.grid_G = tu.G;
     a.z = tu.z;
     a.flags = tu.flags;
     a.aligned = (reinterpret_cast<uintptr_t>(keys) & 15u) == 0;
+    a.idx_bits = 1; // enough for n - 1
+    while (a.idx_bits < 32 && (n - 1) >> a.idx_bits) ++a.idx_bits;
     a.first_dense = -1; // decided on the device unless the host fixes it
     a.kth_only = out_keys == nullptr;
     return a;
 }
 
-// Host copy of the device pivot-rank rule, for sizing buffers and predicting
-// the number of grid levels.
+// Host copy of the device pivot-rank rule, for sizing buffers.
 static double est_bracket(u64 m, u64 k_rem, u32 s, float z) {
     const double kept = (double)std::min<u64>(s, m);
     const double mu_le = kept * (double)k_rem / (double)m;
@@ -1046,11 +868,10 @@ template <int DT> static topk_status set_smem_attrs() {
         cudaFuncSetAttribute(k_pass_tma<DT, PM_COUNT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)TmaCfg<DT, PM_COUNT>::SMEM) != cudaSuccess)
         return TOPK_ECUDA;
-    const int bytes = (int)sizeof(BlockSmem<Key<DT>::KW>);
-    if (cudaFuncSetAttribute(k_pivots<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)sizeof(PivotSmem<Key<DT>::KW>)) != cudaSuccess)
-        return TOPK_ECUDA;
-    if (cudaFuncSetAttribute(k_finish<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess)
+    if (cudaFuncSetAttribute(k_plan<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sizeof(PlanSmem<Key<DT>::KW>)) != cudaSuccess ||
+        cudaFuncSetAttribute(k_finish<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sizeof(FinSmem<Key<DT>::KW>)) != cudaSuccess)
         return TOPK_ECUDA;
     done_mask.fetch_or(bit);
     return TOPK_OK;
@@ -1112,7 +933,7 @@ static topk_status enqueue_select(topk_ctx* ctx, SelArgs a, const Tuning& tu, in
     const u64 n = a.n, k = a.k;
     if (k == 1 || k == n) {
         if (ctx) profile_pass_begin(ctx, st);
-        const cudaError_t e = launch_dep(k_extreme<DT>, sms * EXT_BLOCKS_PER_SM, EXT_NT, 0, st, a,
+        const cudaError_t e = launch_dep(k_extreme<DT>, sms * EXT_BLOCKS_PER_SM, EXT_NT, 0, st, 1, a,
                                          k == n && n > 1 ? 1 : 0, counter, partials);
         if (e != cudaSuccess) return cuda_status(e);
         if (ctx) {
@@ -1128,54 +949,51 @@ static topk_status enqueue_select(topk_ctx* ctx, SelArgs a, const Tuning& tu, in
     a.first_dense =
         bulk ? (first_level_dense(n, k, tu.sample, tu.z, (tu.flags & TOPK_FLAG_RAW_DELTA) != 0) ? 1 : 0) : -1;
     auto first_pass = [&]() -> cudaError_t {
-        if (!bulk) return launch_dep(k_pass_first<DT>, pass_grid<DT>(sms, true), PASS_NT, 0, st, a);
+        if (!bulk) return launch_dep(k_pass_first<DT>, pass_grid<DT>(sms, true), PASS_NT, 0, st, 1, a);
         if (a.first_dense && a.kth_only)
             return launch_dep(k_pass_tma<DT, PM_COUNT>, tma_grid<DT, PM_COUNT>(sms), TMA_NT,
-                              TmaCfg<DT, PM_COUNT>::SMEM, st, a);
+                              TmaCfg<DT, PM_COUNT>::SMEM, st, 1, a);
         if (a.first_dense)
             return launch_dep(k_pass_tma<DT, PM_DENSE>, tma_grid<DT, PM_DENSE>(sms), TMA_NT,
-                              TmaCfg<DT, PM_DENSE>::SMEM, st, a);
+                              TmaCfg<DT, PM_DENSE>::SMEM, st, 1, a);
         return launch_dep(k_pass_tma<DT, PM_SPARSE>, tma_grid<DT, PM_SPARSE>(sms), TMA_NT,
-                          TmaCfg<DT, PM_SPARSE>::SMEM, st, a);
+                          TmaCfg<DT, PM_SPARSE>::SMEM, st, 1, a);
     };
-    // grid levels until the candidates fit the block finisher's range
-    int levels = 0;
-    {
-        double m = (double)n, kr = (double)k;
-        while (m > tu.G && levels < 8) {
-            m = 1.2 * est_bracket((u64)m, (u64)std::max(1.0, std::min(kr, m)), tu.sample, tu.z);
-            kr = m / 2;
-            ++levels;
-        }
-    }
-    const size_t smem = sizeof(BlockSmem<KW>);
-    const int smp_blocks = (int)((tu.sample * SMP_MAX_SCALE + SMP_NT * SMP_DRAWS - 1) / (SMP_NT * SMP_DRAWS));
-    for (int l = 0; l < levels; ++l) {
-        cudaError_t e = launch_dep(k_sample<DT>, smp_blocks, SMP_NT, 0, st, a, l == 0 ? 1 : 0);
-        if (e == cudaSuccess) e = launch_dep(k_pivots<DT>, 1, PIV_NT, sizeof(PivotSmem<KW>), st, a, l == 0 ? 1 : 0);
+    const bool one = n <= tu.T;
+    cudaError_t e = cudaSuccess;
+    if (!one) {
+        // (the finish holds CL_BLOCKS times as many, but a second pass over more
+        // than these takes less time)
+        a.list_max = Lim<KW>::ELEMS;
+        // the bins are kept where they are likely to be needed
+        if (1.2 * est_bracket(n, k, tu.sample, tu.z) <= (double)a.list_max && !(tu.flags & TOPK_FLAG_RAW_DELTA))
+            a.bins = nullptr;
+        e = launch_dep(k_plan<DT>, CL_BLOCKS, CL_NT, sizeof(PlanSmem<KW>), st, CL_BLOCKS, a);
         if (e != cudaSuccess) return cuda_status(e);
-        if (l == 0 && ctx) profile_pass_begin(ctx, st);
-        if (l == 0) e = first_pass();
-        else e = launch_dep(k_pass<DT>, pass_grid<DT>(sms, false), PASS_NT, 0, st, a);
+        if (ctx) profile_pass_begin(ctx, st);
+        e = first_pass();
         if (e != cudaSuccess) return cuda_status(e);
-        if (l == 0 && ctx) profile_pass_end(ctx, st);
+        if (ctx) profile_pass_end(ctx, st);
+        e = launch_dep(k_pass<DT>, pass_grid<DT>(sms, false), PASS_NT, 0, st, 1, a);
+        if (e != cudaSuccess) return cuda_status(e);
     }
-    const cudaError_t e = launch_dep(k_finish<DT>, 1, BLK_NT, smem, st, a, levels == 0 ? 1 : 0);
+    const int fin = one && n <= FIN_SOLO ? 1 : CL_BLOCKS; // (the kernel leaves a short source to one block)
+    e = launch_dep(k_finish<DT>, fin, CL_NT, sizeof(FinSmem<KW>), st, fin, a, one ? 1 : 0);
     if (e != cudaSuccess) return cuda_status(e);
-    if (ctx) count_launch(ctx, 3 * (uint64_t)levels + 1);
+    if (ctx) count_launch(ctx, one ? 1 : 4);
     return cuda_status(cudaGetLastError());
 }
 
-// Scratch regions of one selection: reduction partials, the sample, and the
+// Scratch regions of one selection: reduction partials, the candidates' bins and the
 // two candidate buffers (keys, then positions) of `cap` pairs each.
 struct SelectCarve {
-    size_t part, samp, k0, k1, i0, i1;
+    size_t part, bins, k0, k1, i0, i1;
 };
 template <int KW> static Carve select_carve(u64 cap, int sms, SelectCarve& sc) {
     const size_t kbytes = KW / 8;
     Carve cv;
     sc.part = cv.take(sizeof(typename Comp<KW>::t) * (size_t)sms * EXT_BLOCKS_PER_SM);
-    sc.samp = cv.take(sizeof(typename Comp<KW>::t) * (size_t)Lim<KW>::ELEMS);
+    sc.bins = cv.take(sizeof(LevelBins));
     sc.k0 = cv.take(cap * kbytes);
     sc.k1 = cv.take(cap * kbytes);
     sc.i0 = cv.take(cap * 4);
@@ -1197,14 +1015,12 @@ topk_status run_select(topk_ctx* ctx, const void* keys, u64 n, u64 k, void* out_
     a.cap_b = cap;
     SelectCarve sc;
     const Carve cv = select_carve<KW>(cap, ctx->sms, sc);
-    const size_t off_part = sc.part, off_samp = sc.samp, off_k0 = sc.k0, off_k1 = sc.k1, off_i0 = sc.i0,
+    const size_t off_part = sc.part, off_bins = sc.bins, off_k0 = sc.k0, off_k1 = sc.k1, off_i0 = sc.i0,
                  off_i1 = sc.i1;
     topk_status rs = ensure_scratch(ctx, cv.off);
     if (rs != TOPK_OK) return rs;
     char* base = static_cast<char*>(ctx->scratch.base);
-    a.samp = base + off_samp;
-    a.samp_cap = Lim<KW>::ELEMS;
-    a.samp_count = ctx->d_counter + 3;
+    a.bins = reinterpret_cast<LevelBins*>(base + off_bins);
     a.pass_done = ctx->d_counter + 2;
     a.cand_key[0] = base + off_k0;
     a.cand_key[1] = base + off_k1;
@@ -1215,8 +1031,8 @@ topk_status run_select(topk_ctx* ctx, const void* keys, u64 n, u64 k, void* out_
 
 // ------------------------------------------ entry point without allocation
 // topk_select_noalloc runs the same kernels as topk_select, with every piece
-// of scratch (state, error word, block-done counter, reduction partials and
-// the two candidate buffers) in one file-scope device array instead of a
+// of scratch (state, error word, block-done counters, reduction partials, bins
+// and the two candidate buffers) in one file-scope device array instead of a
 // context's cudaMalloc'd block.  The array lives in every GPU that loads the
 // library until the process exits.  Host code must not pass the array's name
 // to a kernel (in host code it is only a stand-in for the symbol); its device
@@ -1231,12 +1047,11 @@ constexpr u64 NOALLOC_MAX_N = 1ull << 22;  // largest n accepted (4 Mi keys)
 // than the same call through a context; the set-up checks this relation.
 constexpr u64 NOALLOC_CAP = 1ull << 19;
 constexpr size_t NA_OFF_STATE = 0;         // SelState
-constexpr size_t NA_OFF_WORDS = 4096;      // [0] error, [1] reduction done, [2] pass done, [3] sample count
+constexpr size_t NA_OFF_WORDS = 4096;      // [0] error, [1] reduction done, [2] pass done
 constexpr size_t NA_OFF_PART = 8192;       // per-block composites of the k = 1 / k = n reduction
 constexpr size_t NA_PART_BYTES = 64 * 1024;
-constexpr size_t NA_OFF_SAMP = NA_OFF_PART + NA_PART_BYTES; // sample, Lim<32>::ELEMS * 8 = Lim<64>::ELEMS * 16 bytes
-constexpr size_t NA_SAMP_BYTES = 128 * 1024;
-constexpr size_t NA_OFF_CAND = NA_OFF_SAMP + NA_SAMP_BYTES;
+constexpr size_t NA_OFF_BINS = NA_OFF_PART + NA_PART_BYTES; // bins of the first level's candidates
+constexpr size_t NA_OFF_CAND = NA_OFF_BINS + ((sizeof(LevelBins) + 255) & ~(size_t)255);
 constexpr size_t NA_BYTES = NA_OFF_CAND + 2 * NOALLOC_CAP * (8 + 4); // about 12.2 MiB
 
 // Kernel attributes and the launch-geometry queries of every key type, so
@@ -1269,13 +1084,9 @@ topk_status run_select_noalloc(char* base, int sms, const void* keys, u64 n, u64
     a.cand_key[1] = cand + NOALLOC_CAP * 8;
     a.cand_idx[0] = reinterpret_cast<u32*>(cand + 2 * NOALLOC_CAP * 8);
     a.cand_idx[1] = reinterpret_cast<u32*>(cand + 2 * NOALLOC_CAP * 8 + NOALLOC_CAP * 4);
-    static_assert(sizeof(typename Comp<KW>::t) * Lim<KW>::ELEMS <= NA_SAMP_BYTES, "sample region too small");
-    a.samp = base + NA_OFF_SAMP;
-    a.samp_cap = Lim<KW>::ELEMS;
+    a.bins = reinterpret_cast<LevelBins*>(base + NA_OFF_BINS);
     a.pass_done = words + 2;
-    a.samp_count = words + 3;
-    // the error word, the block-done counters and the sample count must
-    // start at zero (a call that failed may have left them set)
+    // the error word and the block-done counters must start at zero (a call that failed may have left them set)
     if (cudaMemsetAsync(words, 0, 4 * sizeof(u32), st) != cudaSuccess) return TOPK_ECUDA;
     if (d_status && cudaMemsetAsync(d_status, 0, sizeof(u32), st) != cudaSuccess) return TOPK_ECUDA;
     return enqueue_select<DT>(nullptr, a, tu, sms, words + 1, base + NA_OFF_PART, st);
