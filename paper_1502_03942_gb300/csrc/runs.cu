@@ -8,16 +8,17 @@
 // hi_r on are known not to be.  Initially hi_r = min(len_r, k): only the
 // first k objects of each run can be selected (Appendix A).
 //
-// One round (k_runs_round, one block per pivot):
+// One round (k_runs_round, one warp per run):
 //   - pivot v_j is drawn uniformly from the undecided objects (a prefix sum
 //     over the bracket sizes locates it, Appendix A);
 //   - every run counts its bracket objects below v_j by binary search
-//     ("find j such that s[1..j] < v", Appendix A), the block sums them into
-//     the pivot's rank (the paper's sum reduction);
+//     ("find j such that s[1..j] < v", Appendix A), and the counts of all runs
+//     are summed into the pivot's rank (the paper's sum reduction);
 //   - the last block to finish (block-done counter, no waiting) keeps the
 //     highest pivot below rank k and the lowest above it, narrows every
 //     bracket and draws the next pivots; a pivot of rank exactly k ends the
 //     search.
+// A flexible round (k_runs_trials) has one block per trial instead.
 // When at most T objects remain undecided, k_runs_finish gathers them into
 // one block, selects the remaining rank among them and derives the splits.
 #include <algorithm>
@@ -33,6 +34,7 @@ constexpr int RUN_NT = 256;
 constexpr int RUN_FIN_NT = 1024;
 constexpr u32 RUN_T = 8192;         // objects finished in one block
 constexpr u32 RUN_MAX_D = 256;      // pivots per round
+constexpr u32 RUN_PREFIX = 4096;    // runs whose bracket prefix is kept in shared memory for the searches
 constexpr u32 RUN_MAX_BLOCK_ROUNDS = 512;
 
 enum : u32 { RPH_RUN = 0, RPH_FINISH = 1, RPH_DONE = 2, RPH_ERROR = 3 };
@@ -58,11 +60,12 @@ struct RunsArgs {
     u64* lo;        // p
     u64* hi;        // p
     u64* prefix;    // p + 1: exclusive prefix of hi - lo
-    u32* cnt;       // d * p: bracket objects of run r below pivot j
+    u32* cnt;       // d * p: bracket objects of run r below pivot j, at j * cj + r * cr
+    u64 cj, cr;
     u64* piv_key;   // d
     u64* piv_g;     // d: concatenated index
     u32* piv_run;   // d
-    u64* piv_rank;  // d: undecided objects below pivot j
+    u64* piv_rank;  // d: undecided objects below pivot j (zero between rounds)
     RunsState* st;
     u32* counter;   // block-done counter (zero between rounds)
     u32* err;
@@ -103,58 +106,92 @@ __device__ __forceinline__ u64 count_below(const u64* keys, u64 base, u64 lo, u6
     return lo;
 }
 
-// Block-wide exclusive prefix of (hi_r - lo_r) into a.prefix; returns the total.
-__device__ u64 block_prefix_brackets(const RunsArgs& a, u64* warp_sums, u64* carry_smem) {
+struct RunsSmem {
+    u64 warp_sums[RUN_FIN_NT / 32 + 1];
+    u64 carry;
+    u64 red[RUN_FIN_NT / 32], red2[RUN_FIN_NT / 32];
+    u32 red3[RUN_FIN_NT / 32];
+    u32 prefix[RUN_PREFIX + 1]; // copy of the prefix when there are at most RUN_PREFIX runs
+    int best_lo, best_hi, exact;
+    u32 flag;
+};
+
+// Block-wide exclusive prefix of (hi_r - lo_r) into a.prefix (and sm.prefix);
+// returns the total.  Four runs per thread and step.
+__device__ u64 block_prefix_brackets(const RunsArgs& a, RunsSmem& sm) {
     const u32 tid = threadIdx.x, lane = lane_id(), warp = tid >> 5, nw = blockDim.x >> 5;
-    if (tid == 0) *carry_smem = 0;
-    __syncthreads();
-    for (u32 base = 0; base < a.p; base += blockDim.x) {
-        const u32 r = base + tid;
-        const u64 v = r < a.p ? a.hi[r] - a.lo[r] : 0;
-        u64 incl = v;
+    const bool keep = a.p <= RUN_PREFIX;
+    u64 carry = 0;
+    for (u32 base = 0; base < a.p; base += 4 * blockDim.x) {
+        u64 v[4], sum = 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const u32 r = base + 4 * tid + q;
+            v[q] = r < a.p ? a.hi[r] - a.lo[r] : 0;
+            sum += v[q];
+        }
+        u64 incl = sum;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const u64 y = __shfl_up_sync(0xffffffffu, incl, o);
             if (lane >= (u32)o) incl += y;
         }
-        if (lane == 31) warp_sums[warp] = incl;
+        __syncthreads(); // (earlier readers of warp_sums)
+        if (lane == 31) sm.warp_sums[warp] = incl;
         __syncthreads();
-        if (tid == 0) {
-            u64 acc = 0;
-            for (u32 w = 0; w < nw; ++w) {
-                const u64 t = warp_sums[w];
-                warp_sums[w] = acc;
-                acc += t;
-            }
-            warp_sums[nw] = acc;
+        u64 before = 0, all = 0;
+        for (u32 w = 0; w < nw; ++w) {
+            const u64 x = sm.warp_sums[w];
+            before += w < warp ? x : 0;
+            all += x;
         }
-        __syncthreads();
-        const u64 carry = *carry_smem;
-        if (r < a.p) a.prefix[r] = carry + warp_sums[warp] + incl - v;
-        __syncthreads();
-        if (tid == 0) *carry_smem = carry + warp_sums[nw];
-        __syncthreads();
+        u64 at = carry + before + incl - sum;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const u32 r = base + 4 * tid + q;
+            if (r < a.p) {
+                a.prefix[r] = at;
+                if (keep) sm.prefix[r] = (u32)at;
+            }
+            at += v[q];
+        }
+        carry += all;
     }
-    const u64 total = *carry_smem;
-    if (tid == 0) a.prefix[a.p] = total;
+    if (tid == 0) {
+        a.prefix[a.p] = carry;
+        if (keep) sm.prefix[a.p] = (u32)carry; // (at most 2^32 - 1 objects)
+    }
     __syncthreads();
-    return total;
+    return carry;
 }
 
-// Draws the d pivots of round `round` uniformly among the m undecided
-// objects (prefix must be current).
-__device__ void draw_pivots(const RunsArgs& a, u64 m, u32 round) {
-    for (u32 j = threadIdx.x; j < a.d; j += blockDim.x) {
-        const Philox4 rr = philox4x32_10(j, round, 0x52554E53u, 0, (u32)a.seed, (u32)(a.seed >> 32));
-        const u64 u64r = ((u64)rr.v[1] << 32) | rr.v[0];
-        const u64 u = (u64)(((u128)u64r * m) >> 64); // uniform in [0, m)
-        // run r with prefix[r] <= u < prefix[r+1]
-        u32 lo = 0, hi = a.p;
+// The run r with prefix[r] <= u < prefix[r + 1] (both copies current).
+__device__ __forceinline__ u32 run_of(const RunsArgs& a, const RunsSmem& sm, u64 u) {
+    u32 lo = 0, hi = a.p;
+    if (a.p <= RUN_PREFIX) {
+        while (hi - lo > 1) {
+            const u32 mid = (lo + hi) / 2;
+            if (sm.prefix[mid] <= (u32)u) lo = mid;
+            else hi = mid;
+        }
+    } else {
         while (hi - lo > 1) {
             const u32 mid = (lo + hi) / 2;
             if (a.prefix[mid] <= u) lo = mid;
             else hi = mid;
         }
+    }
+    return lo;
+}
+
+// Draws the d pivots of round `round` uniformly among the m undecided
+// objects (prefix must be current).
+__device__ void draw_pivots(const RunsArgs& a, const RunsSmem& sm, u64 m, u32 round) {
+    for (u32 j = threadIdx.x; j < a.d; j += blockDim.x) {
+        const Philox4 rr = philox4x32_10(j, round, 0x52554E53u, 0, (u32)a.seed, (u32)(a.seed >> 32));
+        const u64 u64r = ((u64)rr.v[1] << 32) | rr.v[0];
+        const u64 u = (u64)(((u128)u64r * m) >> 64); // uniform in [0, m)
+        const u32 lo = run_of(a, sm, u);
         const u64 pos = a.lo[lo] + (u - a.prefix[lo]);
         const u64 g = a.off[lo] + pos;
         a.piv_key[j] = a.keys[g];
@@ -292,48 +329,60 @@ __device__ void draw_flexible_block(const RunsArgs& a, const RunsState& st, u32 
     __syncthreads();
 }
 
-struct RunsSmem {
-    u64 warp_sums[RUN_FIN_NT / 32 + 1];
-    u64 carry;
-    u64 red[RUN_FIN_NT / 32];
-    int best_lo, best_hi, exact;
-    u32 flag;
-};
-
 // The branch after a round: keep the tightest pivots (one block).
 __device__ void runs_decide(const RunsArgs& a, RunsSmem& sm) {
     RunsState* st = a.st;
     const u32 tid = threadIdx.x;
-    if (tid == 0) {
-        // the undecided objects below the pivot sought: exactly k_rem - 1, or
-        // (flexible) any number in [kmin - 1, kmax - 1]
-        const u64 tlo = a.flexible ? st->kmin - 1 : st->k_rem - 1;
-        const u64 thi = a.flexible ? st->kmax - 1 : st->k_rem - 1;
-        int bl = -1, bh = -1, ex = -1;
-        u64 rl = 0, rh = ~(u64)0;
-        for (u32 j = 0; j < a.d; ++j) {
-            if (__ldcg(a.piv_g + j) == VOID_PIVOT) continue;
-            const u64 rj = __ldcg(a.piv_rank + j);
-            if (rj >= tlo && rj <= thi) {
-                if (ex < 0) ex = (int)j;
-            } else if (rj < tlo && (bl < 0 || rj > rl)) {
-                bl = (int)j;
-                rl = rj;
-            } else if (rj > thi && (bh < 0 || rj < rh)) {
-                bh = (int)j;
-                rh = rj;
-            }
+    // the undecided objects below the pivot sought: exactly k_rem - 1, or
+    // (flexible) any number in [kmin - 1, kmax - 1]; of equally good pivots the
+    // first.  One pivot per thread and step, then a reduction over the block.
+    const u64 tlo = a.flexible ? st->kmin - 1 : st->k_rem - 1;
+    const u64 thi = a.flexible ? st->kmax - 1 : st->k_rem - 1;
+    u64 below = 0, above = ~(u64)0; // (rank + 1, descending pivot number); (rank, pivot number)
+    u32 hit = 0xFFFFFFFFu;
+    for (u32 j = tid; j < a.d; j += blockDim.x) {
+        if (__ldcg(a.piv_g + j) == VOID_PIVOT) continue;
+        const u64 rj = __ldcg(a.piv_rank + j);
+        if (rj >= tlo && rj <= thi) {
+            hit = hit < j ? hit : j;
+        } else if (rj < tlo) {
+            const u64 w = ((rj + 1) << 9) | (511u - j);
+            below = w > below ? w : below;
+        } else {
+            const u64 w = (rj << 9) | j;
+            above = w < above ? w : above;
         }
-        sm.best_lo = bl;
-        sm.best_hi = bh;
-        sm.exact = ex;
+    }
+    static_assert(RUN_MAX_D <= 512, "a pivot number takes 9 bits");
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const u64 b2 = __shfl_xor_sync(0xffffffffu, below, o), a2 = __shfl_xor_sync(0xffffffffu, above, o);
+        below = b2 > below ? b2 : below;
+        above = a2 < above ? a2 : above;
+    }
+    hit = __reduce_min_sync(0xffffffffu, hit);
+    if (lane_id() == 0) {
+        sm.red[tid >> 5] = below;
+        sm.red2[tid >> 5] = above;
+        sm.red3[tid >> 5] = hit;
+    }
+    __syncthreads();
+    if (tid == 0) {
+        for (u32 w = 1; w < blockDim.x / 32; ++w) {
+            below = sm.red[w] > below ? sm.red[w] : below;
+            above = sm.red2[w] < above ? sm.red2[w] : above;
+            hit = sm.red3[w] < hit ? sm.red3[w] : hit;
+        }
+        sm.best_lo = below ? (int)(511u - (u32)(below & 511u)) : -1;
+        sm.best_hi = above != ~(u64)0 ? (int)(above & 511u) : -1;
+        sm.exact = hit != 0xFFFFFFFFu ? (int)hit : -1;
     }
     __syncthreads();
     const int ex = sm.exact, bl = sm.best_lo, bh = sm.best_hi;
     if (ex >= 0) { // pivot ex has rank k: everything below it is selected
         const u32 vr = a.piv_run[ex];
         for (u32 r = tid; r < a.p; r += blockDim.x)
-            a.split[r] = a.lo[r] + __ldcg(a.cnt + (size_t)ex * a.p + r) + (r == vr ? 1 : 0);
+            a.split[r] = a.lo[r] + __ldcg(a.cnt + ex * a.cj + r * a.cr) + (r == vr ? 1 : 0);
         if (tid == 0) {
             *a.kth_key = a.piv_key[ex];
             *a.kth_run = vr;
@@ -346,11 +395,11 @@ __device__ void runs_decide(const RunsArgs& a, RunsSmem& sm) {
     }
     for (u32 r = tid; r < a.p; r += blockDim.x) {
         const u64 l = a.lo[r];
-        if (bh >= 0) a.hi[r] = l + __ldcg(a.cnt + (size_t)bh * a.p + r);
-        if (bl >= 0) a.lo[r] = l + __ldcg(a.cnt + (size_t)bl * a.p + r) + (r == a.piv_run[bl] ? 1 : 0);
+        if (bh >= 0) a.hi[r] = l + __ldcg(a.cnt + bh * a.cj + r * a.cr);
+        if (bl >= 0) a.lo[r] = l + __ldcg(a.cnt + bl * a.cj + r * a.cr) + (r == a.piv_run[bl] ? 1 : 0);
     }
     __syncthreads();
-    const u64 m = block_prefix_brackets(a, sm.warp_sums, &sm.carry);
+    const u64 m = block_prefix_brackets(a, sm);
     if (tid == 0) {
         if (bl >= 0) {
             const u64 below = __ldcg(a.piv_rank + bl) + 1; // now selected
@@ -370,8 +419,9 @@ __device__ void runs_decide(const RunsArgs& a, RunsSmem& sm) {
         if (m <= RUN_T) st->phase = RPH_FINISH;
     }
     __syncthreads();
+    for (u32 j = tid; j < a.d; j += blockDim.x) a.piv_rank[j] = 0; // for the next round
     // (flexible trials are drawn by the next round's blocks, one per trial)
-    if (st->phase == RPH_RUN && !a.flexible) draw_pivots(a, m, st->round);
+    if (st->phase == RPH_RUN && !a.flexible) draw_pivots(a, sm, m, st->round);
     __syncthreads();
 }
 
@@ -411,7 +461,7 @@ __global__ void __launch_bounds__(RUN_FIN_NT) k_runs_init(RunsArgs a) {
         if (e < s || c > len) runs_latch(a, ST_EINVAL);
     }
     __syncthreads();
-    const u64 m = block_prefix_brackets(a, sm.warp_sums, &sm.carry);
+    const u64 m = block_prefix_brackets(a, sm);
     if (threadIdx.x == 0) {
         st->m = m;
         // (m holds every remaining object when fewer than k remain in total)
@@ -420,7 +470,8 @@ __global__ void __launch_bounds__(RUN_FIN_NT) k_runs_init(RunsArgs a) {
         if (st->phase == RPH_RUN && m <= RUN_T) st->phase = RPH_FINISH;
     }
     __syncthreads();
-    if (st->phase == RPH_RUN && !a.flexible) draw_pivots(a, m, 0);
+    for (u32 j = threadIdx.x; j < a.d; j += blockDim.x) a.piv_rank[j] = 0;
+    if (st->phase == RPH_RUN && !a.flexible) draw_pivots(a, sm, m, 0);
 }
 
 // Optional order check: every run non-decreasing (one block per run).
@@ -436,8 +487,103 @@ __global__ void __launch_bounds__(RUN_NT) k_runs_check_sorted(RunsArgs a) {
         }
 }
 
-// One pivot per block: rank of v_j among the undecided objects.
+// Ranks of the d pivots among the undecided objects, one warp per run: each
+// lane searches the run for up to eight pivots at once, in steps that are the
+// same for all (the interval's length is halved whatever the comparison says),
+// so a lane's loads are in flight together, and the upper levels of a run's
+// search tree, which all pivots share, are read by one warp.  Bound by the
+// latency of the dependent loads (about log2 of the bracket) and, with many
+// pivots, by their number: 1024 runs of 2^U(10, 20) keys, k = half of them, take
+// 58 us with the 64 pivots of a round, 64 us with 128 and 90 us with 256 (one round
+// fewer) on keys that lie in L2; one block per pivot, whose threads walked four
+// runs one after the other, took 155 us.
+constexpr u32 RUN_PER_LANE = RUN_MAX_D / 32;
+
+template <int PL>
+__device__ __forceinline__ void rank_pivots(const RunsArgs& a, const u64* pk, const u32* pg, u32* rank_smem) {
+    const u32 lane = lane_id(), warp = threadIdx.x >> 5;
+    const u32 warps = gridDim.x * (RUN_NT / 32);
+    u64 vk[PL];
+    u32 vg[PL], acc[PL];
+#pragma unroll
+    for (int q = 0; q < PL; ++q) {
+        const u32 j = q * 32 + lane;
+        vk[q] = j < a.d ? pk[j] : 0;
+        vg[q] = j < a.d ? pg[j] : 0;
+        acc[q] = 0;
+    }
+    for (u32 r = blockIdx.x * (RUN_NT / 32) + warp; r < a.p; r += warps) {
+        const u32 first = (u32)(a.off[r] + a.lo[r]); // positions are below 2^32
+        u32 n = (u32)(a.hi[r] - a.lo[r]);
+        u32 at[PL]; // objects below the pivot found so far
+#pragma unroll
+        for (int q = 0; q < PL; ++q) at[q] = 0;
+        while (n > 0) {
+            const u32 half = (n + 1) / 2; // objects 0..half-1 of the interval lie below the pivot iff the last does
+            u64 key[PL];
+#pragma unroll
+            for (int q = 0; q < PL; ++q) key[q] = __ldg(a.keys + (first + at[q] + half - 1));
+#pragma unroll
+            for (int q = 0; q < PL; ++q) {
+                const u32 g = first + at[q] + half - 1;
+                if (key[q] < vk[q] || (key[q] == vk[q] && g < vg[q])) at[q] += half;
+            }
+            n -= half;
+        }
+#pragma unroll
+        for (int q = 0; q < PL; ++q) {
+            const u32 j = q * 32 + lane;
+            if (j < a.d) a.cnt[j * a.cj + r * a.cr] = at[q];
+            acc[q] += at[q];
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < PL; ++q) {
+        const u32 j = q * 32 + lane;
+        if (j < a.d && acc[q]) atomicAdd(&rank_smem[j], acc[q]);
+    }
+}
+
 __global__ void __launch_bounds__(RUN_NT) k_runs_round(RunsArgs a) {
+    grid_dep_wait();
+    grid_dep_release();
+    __shared__ RunsSmem sm;
+    __shared__ u64 pk[RUN_MAX_D];
+    __shared__ u32 pg[RUN_MAX_D], rank[RUN_MAX_D];
+    __shared__ u32 is_last;
+    static_assert(RUN_NT >= (int)RUN_MAX_D, "one thread per pivot");
+    RunsState* st = a.st;
+    if (st->phase != RPH_RUN) return;
+    if (threadIdx.x < a.d) {
+        pk[threadIdx.x] = a.piv_key[threadIdx.x];
+        pg[threadIdx.x] = (u32)a.piv_g[threadIdx.x];
+        rank[threadIdx.x] = 0;
+    }
+    __syncthreads();
+    if (a.d <= 32) rank_pivots<1>(a, pk, pg, rank);
+    else if (a.d <= 64) rank_pivots<2>(a, pk, pg, rank);
+    else if (a.d <= 128) rank_pivots<4>(a, pk, pg, rank);
+    else rank_pivots<RUN_PER_LANE>(a, pk, pg, rank);
+    __syncthreads();
+    if (threadIdx.x < a.d && rank[threadIdx.x])
+        atomicAdd(reinterpret_cast<unsigned long long*>(a.piv_rank + threadIdx.x), (unsigned long long)rank[threadIdx.x]);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        is_last = atomicAdd(a.counter, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!is_last) return;
+    __threadfence();
+    if (threadIdx.x == 0) {
+        *a.counter = 0;
+        st->rounds_grid += 1;
+    }
+    runs_decide(a, sm);
+}
+
+// A flexible round: one trial per block, drawn and ranked by it.
+__global__ void __launch_bounds__(RUN_NT) k_runs_trials(RunsArgs a) {
     grid_dep_wait();
     grid_dep_release();
     __shared__ RunsSmem sm;
@@ -447,14 +593,14 @@ __global__ void __launch_bounds__(RUN_NT) k_runs_round(RunsArgs a) {
     RunsState* st = a.st;
     if (st->phase != RPH_RUN) return;
     const u32 j = blockIdx.x;
-    if (a.flexible) draw_flexible_block(a, *st, j, st->round, red_k, red_g, red_r);
+    draw_flexible_block(a, *st, j, st->round, red_k, red_g, red_r);
     const u64 vk = a.piv_key[j], vg = a.piv_g[j];
     u64 acc = 0;
     if (vg != VOID_PIVOT) // (a void trial has no estimate to rank)
         for (u32 r = threadIdx.x; r < a.p; r += blockDim.x) {
             const u64 lo = a.lo[r], hi = a.hi[r], base = a.off[r];
             const u64 c = count_below(a.keys, base, lo, hi, vk, vg) - lo;
-            a.cnt[(size_t)j * a.p + r] = (u32)c;
+            a.cnt[j * a.cj + r * a.cr] = (u32)c;
             acc += c;
         }
 #pragma unroll
@@ -489,7 +635,7 @@ __global__ void __launch_bounds__(RUN_FIN_NT) k_runs_finish(RunsArgs a) {
     ct* items = reinterpret_cast<ct*>(smem_raw);                    // RUN_T composites
     u32* run_cnt = reinterpret_cast<u32*>(items + RUN_T);          // per-run selected counts (chunked)
     __shared__ RunsSmem sm;
-    __shared__ RadixSmem<64, 1> rs;
+    __shared__ HistSelSmem<64> hs;
     RunsState* st = a.st;
     for (u32 it = 0; it < RUN_MAX_BLOCK_ROUNDS && st->phase == RPH_RUN; ++it) {
         if (a.flexible) {
@@ -502,7 +648,7 @@ __global__ void __launch_bounds__(RUN_FIN_NT) k_runs_finish(RunsArgs a) {
             for (u32 r = threadIdx.x; r < a.p && vg != VOID_PIVOT; r += blockDim.x) {
                 const u64 lo = a.lo[r];
                 const u64 c = count_below(a.keys, a.off[r], lo, a.hi[r], vk, vg) - lo;
-                a.cnt[(size_t)j * a.p + r] = (u32)c;
+                a.cnt[j * a.cj + r * a.cr] = (u32)c;
                 acc += c;
             }
 #pragma unroll
@@ -525,17 +671,33 @@ __global__ void __launch_bounds__(RUN_FIN_NT) k_runs_finish(RunsArgs a) {
         return;
     }
     if (st->phase != RPH_FINISH) return; // done by an exact pivot, or error
-    // gather the undecided objects (prefix is current)
+    // gather the undecided objects (a.prefix is current), at most RUN_T / RUN_FIN_NT
+    // per thread, whose runs it remembers for the splits
+    constexpr u32 OWN = RUN_T / RUN_FIN_NT;
     const u64 m = st->m;
-    for (u64 i = threadIdx.x; i < m; i += blockDim.x) {
-        u32 lo = 0, hi = a.p;
-        while (hi - lo > 1) {
-            const u32 mid = (lo + hi) / 2;
-            if (a.prefix[mid] <= i) lo = mid;
-            else hi = mid;
-        }
-        const u64 g = a.off[lo] + a.lo[lo] + (i - a.prefix[lo]);
-        items[i] = C::make(a.keys[g], (u32)g);
+    if (a.p <= RUN_PREFIX)
+        for (u32 r = threadIdx.x; r <= a.p; r += blockDim.x) sm.prefix[r] = (u32)a.prefix[r];
+    __syncthreads();
+    u32 own_run[OWN];
+    ct mn = ~(ct)0, mx = 0;
+#pragma unroll
+    for (u32 q = 0; q < OWN; ++q) {
+        const u64 i = threadIdx.x + (u64)q * RUN_FIN_NT;
+        own_run[q] = 0;
+        if (i >= m) continue;
+        const u32 r = run_of(a, sm, i);
+        const u64 g = a.off[r] + a.lo[r] + (i - a.prefix[r]);
+        own_run[q] = r;
+        const ct c = C::make(a.keys[g], (u32)g);
+        items[i] = c;
+        mn = c < mn ? c : mn;
+        mx = c > mx ? c : mx;
+    }
+    // their range by leading words
+    const u32 wmn = __reduce_min_sync(0xffffffffu, (u32)(mn >> 64)), wmx = __reduce_max_sync(0xffffffffu, (u32)(mx >> 64));
+    if (lane_id() == 0) {
+        sm.red3[threadIdx.x >> 5] = wmn;
+        sm.red[threadIdx.x >> 5] = wmx;
     }
     __syncthreads();
     const u32 count = (u32)m;
@@ -543,9 +705,13 @@ __global__ void __launch_bounds__(RUN_FIN_NT) k_runs_finish(RunsArgs a) {
         if (threadIdx.x == 0) runs_latch(a, ST_EINTERNAL);
         return;
     }
-    const u32 rk[1] = {(u32)(st->k_rem - 1)};
-    block_select_ranks<64, 1>(items, count, rk, rs);
-    const ct kth = rs.result[0];
+    u32 lead_lo = 0xFFFFFFFFu, lead_hi = 0;
+    for (u32 w = 0; w < RUN_FIN_NT / 32; ++w) {
+        lead_lo = min(lead_lo, sm.red3[w]);
+        lead_hi = max(lead_hi, (u32)sm.red[w]);
+    }
+    const ct kth = block_select_hist<64, RUN_FIN_NT>(items, count, (ct)lead_lo << 64,
+                                                    ((ct)lead_hi << 64) | (((ct)1 << 64) - 1), (u32)(st->k_rem - 1), hs);
     const u32 kg = C::idx(kth);
     // run of the rank-k object
     if (threadIdx.x == 0) {
@@ -568,17 +734,10 @@ __global__ void __launch_bounds__(RUN_FIN_NT) k_runs_finish(RunsArgs a) {
         const u32 nr = min((u32)RUN_FIN_NT, a.p - r0);
         for (u32 r = threadIdx.x; r < nr; r += blockDim.x) run_cnt[r] = 0;
         __syncthreads();
-        for (u32 i = threadIdx.x; i < count; i += blockDim.x) {
-            const ct c = items[i];
-            if (c > kth) continue;
-            // run of item i by its rank among the brackets (prefix)
-            u32 lo = 0, hi = a.p;
-            while (hi - lo > 1) {
-                const u32 mid = (lo + hi) / 2;
-                if (a.prefix[mid] <= i) lo = mid;
-                else hi = mid;
-            }
-            if (lo >= r0 && lo < r0 + nr) atomicAdd(&run_cnt[lo - r0], 1u);
+#pragma unroll
+        for (u32 q = 0; q < OWN; ++q) {
+            const u32 i = threadIdx.x + q * RUN_FIN_NT, r = own_run[q];
+            if (i < count && items[i] <= kth && r >= r0 && r < r0 + nr) atomicAdd(&run_cnt[r - r0], 1u);
         }
         __syncthreads();
         for (u32 r = threadIdx.x; r < nr; r += blockDim.x) a.split[r0 + r] = a.lo[r0 + r] + run_cnt[r];
@@ -588,8 +747,9 @@ __global__ void __launch_bounds__(RUN_FIN_NT) k_runs_finish(RunsArgs a) {
 }
 
 static u32 runs_rounds_for(u64 p, u64 k, u32 d) {
-    // undecided objects start at most p*k and shrink by about d/2 per round
-    double m = (double)p * (double)k;
+    // undecided objects start at most p * k, and all objects are fewer than
+    // 2^32; they shrink by about d/2 per round
+    double m = std::min((double)p * (double)k, 4294967295.0);
     const double shrink = std::max(2.0, d / 3.0);
     u32 r = 0;
     while (m > RUN_T && r < 12) {
@@ -654,6 +814,8 @@ static topk_status run_sorted_runs(topk_ctx* ctx, const void* d_keys, const uint
     a.hi = reinterpret_cast<u64*>(base + o_hi);
     a.prefix = reinterpret_cast<u64*>(base + o_pre);
     a.cnt = reinterpret_cast<u32*>(base + o_cnt);
+    a.cj = flexible ? p : 1; // a trial's block, or a run's warp, writes consecutive words
+    a.cr = flexible ? 1 : a.d;
     a.piv_key = reinterpret_cast<u64*>(base + o_pk);
     a.piv_g = reinterpret_cast<u64*>(base + o_pg);
     a.piv_run = reinterpret_cast<u32*>(base + o_pr);
@@ -683,7 +845,10 @@ static topk_status run_sorted_runs(topk_ctx* ctx, const void* d_keys, const uint
     cudaError_t e = launch_dep(k_runs_init, 1, RUN_FIN_NT, 0, st, 1, a);
     if (e == cudaSuccess && (prm.flags & TOPK_FLAG_CHECK_SORTED))
         e = launch_dep(k_runs_check_sorted, (int)p, RUN_NT, 0, st, 1, a);
-    for (u32 r = 0; r < rounds && e == cudaSuccess; ++r) e = launch_dep(k_runs_round, (int)a.d, RUN_NT, 0, st, 1, a);
+    const int warps_grid = (int)std::min<u64>((p + RUN_NT / 32 - 1) / (RUN_NT / 32), (u64)ctx->sms * 4);
+    for (u32 r = 0; r < rounds && e == cudaSuccess; ++r)
+        e = flexible ? launch_dep(k_runs_trials, (int)a.d, RUN_NT, 0, st, 1, a)
+                     : launch_dep(k_runs_round, warps_grid, RUN_NT, 0, st, 1, a);
     if (e == cudaSuccess) e = launch_dep(k_runs_finish, 1, RUN_FIN_NT, fin_smem, st, 1, a);
     if (e != cudaSuccess) return cuda_status(e);
     count_launch(ctx, 2 + rounds + ((prm.flags & TOPK_FLAG_CHECK_SORTED) ? 1 : 0));

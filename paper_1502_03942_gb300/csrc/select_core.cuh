@@ -921,180 +921,6 @@ __device__ void pass_tiles(const Src& src, u64 tile0, u64 tile_step,
     }
 }
 
-// ------------------------------------------------------- radix selection
-// Block-wide selection of the elements of given 0-based ranks among
-// v[0..count) (duplicates counted), by most-significant-digit-first radix
-// selection over 8-bit digits of the composite.  Used to read the pivots off
-// the sample (the sample order statistics of ranks k|S|/n -/+ Delta) and the
-// k-th element off the final candidates.  Equivalent to sorting and indexing.
-//
-// Per digit, every element that still matches a target's prefix is counted
-// into that target's 256-bin histogram.  Lanes of a warp holding the same
-// digit are grouped with eight ballots (one per digit bit), so each distinct
-// digit costs one shared-memory atomic per warp even when all keys tie; warps
-// without a matching element skip the grouping.  A target is resolved as
-// soon as its bin holds a single element.
-
-template <int KW, int NTGT> struct RadixSmem {
-    typedef typename Comp<KW>::t ct;
-    ct diff[32];
-    u32 hist[NTGT][256];
-    ct prefix[NTGT];
-    ct mask[NTGT];
-    u32 rank[NTGT];
-    u32 done[NTGT];
-    u32 unique[NTGT];
-    ct result[NTGT];
-};
-
-// Lanes whose 8-bit `dig` equals this lane's (all 32 lanes call).
-__device__ __forceinline__ u32 warp_same_digit(u32 dig) {
-    u32 same = 0xffffffffu;
-#pragma unroll
-    for (int b = 0; b < 8; ++b) {
-        const u32 bal = __ballot_sync(0xffffffffu, (dig >> b) & 1u);
-        same &= ((dig >> b) & 1u) ? bal : ~bal;
-    }
-    return same;
-}
-
-template <int KW, int NTGT>
-__device__ void block_select_ranks(const typename Comp<KW>::t* v, u32 count, const u32 (&rank)[NTGT],
-                                   RadixSmem<KW, NTGT>& sm) {
-    typedef Comp<KW> C;
-    typedef typename C::t ct;
-    const u32 tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
-    // Leading digits shared by every element need no pass: find the highest
-    // bit in which any element differs from the first one.
-    ct x = 0;
-    if (count > 0) {
-        const ct v0 = v[0];
-        for (u32 i = tid; i < count; i += blockDim.x) x |= v[i] ^ v0;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const u64 lo64 = __shfl_xor_sync(0xffffffffu, (unsigned long long)(u64)x, o);
-        ct y = (ct)lo64;
-        if constexpr (sizeof(ct) > 8) y |= (ct)__shfl_xor_sync(0xffffffffu, (unsigned long long)(u64)((u128)x >> 64), o) << 64;
-        x |= y;
-    }
-    if (lane == 0) sm.diff[warp] = x;
-    __syncthreads();
-    ct diff = 0;
-    for (u32 w = 0; w < (blockDim.x >> 5); ++w) diff |= sm.diff[w];
-    constexpr int TOTAL = C::DIGITS * 8;
-    int d0 = C::DIGITS; // all equal: every target is v[0]
-    if (diff != 0) d0 = (TOTAL - bit_length_fast(diff)) / 8;
-    ct top = 0; // mask of the shared leading digits
-    if (d0 > 0) {
-        const int keep = 8 * (C::DIGITS - (d0 < C::DIGITS ? d0 : C::DIGITS));
-        if constexpr (TOTAL == 64) top = keep >= 64 ? (ct)0 : (ct)(~(u64)0 << keep);
-        else top = (keep >= TOTAL) ? (ct)0 : (ct)(((ct)1 << TOTAL) - 1) & ~(ct)(((ct)1 << keep) - 1);
-    }
-    if (tid < NTGT) {
-        sm.prefix[tid] = count > 0 ? (v[0] & top) : (ct)0;
-        sm.mask[tid] = top;
-        sm.rank[tid] = rank[tid];
-        sm.done[tid] = d0 >= C::DIGITS;
-        sm.unique[tid] = 0;
-    }
-    __syncthreads();
-    for (int d = d0; d < C::DIGITS; ++d) {
-        bool all_done = true;
-#pragma unroll
-        for (int t = 0; t < NTGT; ++t) all_done = all_done && sm.done[t];
-        if (all_done) break; // uniform: every thread reads the same smem
-        for (u32 i = tid; i < NTGT * 256; i += blockDim.x) (&sm.hist[0][0])[i] = 0;
-        __syncthreads();
-        ct pfx[NTGT], msk[NTGT];
-        bool live[NTGT];
-#pragma unroll
-        for (int t = 0; t < NTGT; ++t) {
-            pfx[t] = sm.prefix[t];
-            msk[t] = sm.mask[t];
-            live[t] = !sm.done[t];
-        }
-        for (u32 base = 0; base < count; base += blockDim.x) {
-            const u32 i = base + tid;
-            const bool ok = i < count;
-            const ct c = ok ? v[i] : (ct)0;
-            const u32 dig = C::digit(c, d);
-            bool m[NTGT];
-            bool anym = false;
-#pragma unroll
-            for (int t = 0; t < NTGT; ++t) {
-                m[t] = ok && live[t] && ((c & msk[t]) == pfx[t]);
-                anym = anym || m[t];
-            }
-            if (!__any_sync(0xffffffffu, anym)) continue;
-            const u32 same = warp_same_digit(dig);
-#pragma unroll
-            for (int t = 0; t < NTGT; ++t) {
-                const u32 grp = same & __ballot_sync(0xffffffffu, m[t]);
-                if (m[t] && lane == (u32)(__ffs(grp) - 1)) atomicAdd(&sm.hist[t][dig], (u32)__popc(grp));
-            }
-        }
-        __syncthreads();
-        if (warp < (u32)NTGT && live[warp]) {
-            const int t = warp;
-            u32 h[8], s = 0;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                h[j] = sm.hist[t][lane * 8 + j];
-                s += h[j];
-            }
-            u32 incl = s;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const u32 y = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= (u32)o) incl += y;
-            }
-            const u32 excl = incl - s;
-            const u32 r = sm.rank[t];
-            if (r >= excl && r < incl) {
-                // the bin of this lane's 8 holding rank r, and the count below it
-                u32 acc = excl, hb = 0;
-                int b = -1;
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    if (b < 0) {
-                        if (r < acc + h[j]) {
-                            b = j;
-                            hb = h[j];
-                        } else {
-                            acc += h[j];
-                        }
-                    }
-                }
-                const u32 bin = lane * 8 + b;
-                const int shift = (C::DIGITS - 1 - d) * 8;
-                sm.prefix[t] = pfx[t] | ((ct)bin << shift);
-                sm.mask[t] = msk[t] | ((ct)0xFFu << shift);
-                sm.rank[t] = r - acc;
-                if (hb == 1) {
-                    sm.unique[t] = 1;
-                    sm.done[t] = 1;
-                } else if (d == C::DIGITS - 1) {
-                    sm.done[t] = 1;
-                }
-            }
-        }
-        __syncthreads();
-    }
-    // Targets fixed on every digit are the prefix itself; a target whose bin
-    // held one element is that element.
-    if (tid < NTGT) sm.result[tid] = sm.prefix[tid];
-    __syncthreads();
-#pragma unroll
-    for (int t = 0; t < NTGT; ++t) {
-        if (!sm.unique[t]) continue;
-        const ct msk = sm.mask[t], pfx = sm.prefix[t];
-        for (u32 i = tid; i < count; i += blockDim.x)
-            if ((v[i] & msk) == pfx) sm.result[t] = v[i];
-    }
-    __syncthreads();
-}
-
 // A composite from lane `src` (all 32 lanes call).
 template <class CT> __device__ __forceinline__ CT shfl_comp(CT x, u32 src) {
     CT y = (CT)__shfl_sync(0xffffffffu, (unsigned long long)(u64)x, src);
