@@ -2,18 +2,21 @@
 // uneven length, each with its own k) in one persistent launch.
 //
 // The paper has no batched form; each row is the selection of Section 2
-// (Algorithm "select").  A row up to the split length is selected whole by
-// one thread block: sample, pivots, a block-wide partitioning pass into the
-// block's candidate buffer, the branch, and the exact finish among at most T
-// candidates (select_block.cuh).  A longer ("wide") row takes its first
-// level as topk_select does, over the whole GPU: one block samples the row
-// and picks its pivots (k_wide_plan), one grid-wide pass streams the tiles
-// of all wide rows and classifies each against its own row's pivots, the
-// last block to finish a row taking the branch (k_wide_pass), and the
-// persistent kernel then finishes the wide rows from their candidates while
-// it selects the short rows whole.  Rows are handed out longest first from a
-// device work queue, so the blocks that finish early take the short rows at
-// the end.
+// (Algorithm "select").  A row whose k is small (k_rows) is selected by one
+// thread block in one read: a sample gives an upper pivot, the row is streamed
+// and its elements up to the pivot gathered in shared memory, and the element of
+// rank k among them ends the row.  Every other row takes the general path: up to
+// the split length it is selected whole by one block, by levels of sample,
+// pivots, a partitioning pass into the block's candidate buffer, the branch, and
+// the exact finish among at most T candidates (k_batched, select_block.cuh); a
+// longer ("wide") row takes its first level as topk_select does, over the whole
+// GPU: one block samples the row and picks its pivots (k_wide_plan), one
+// grid-wide pass streams the tiles of all wide rows and classifies each against
+// its own row's pivots, the last block to finish a row taking the branch
+// (k_wide_pass), and the persistent kernel then finishes the wide rows from
+// their candidates while it selects the short rows whole.  Rows are handed out
+// longest first from a device work queue, so the blocks that finish early take
+// the short rows at the end.
 #include <algorithm>
 #include <atomic>
 #include <cstdio>
@@ -73,7 +76,11 @@ struct BatchArgs {
     void* const* row_kth_key;
     u32* const* row_kth_idx;
     u32* order;         // rows: row ids, longest first
-    u32* queue;         // next index into order
+    u32* rest;          // rows left to the general path by k_rows (null: all rows)
+    u32* nrest;         // their number (zero between calls)
+    u32* rows_done;     // blocks of k_rows or k_batched that are done (zero between kernels)
+    u32 ordered;        // k_rows takes the rows in `order` from the queue, else row i in block i
+    u32* queue;         // next index into order (zero between kernels)
     SelState* states;   // one per block
     char* cand;         // per block: key'[2][CAP], idx[2][CAP]
     u64 seed;
@@ -85,7 +92,7 @@ struct BatchArgs {
     u32 key_bytes;      // width of a key
     u32 split;          // rows longer than this are wide
     u32* wide;          // rows: ids of the wide rows, longest first
-    u32* words;         // [0] wide rows, [1] planning queue
+    u32* words;         // [0] wide rows, [1] planning queue, [2] rows in order
     u64* tile_pre;      // rows + 1: tiles of the wide rows before the j-th
     u32* done;          // rows: tiles of the row classified by the wide pass
     SelState* rstate;   // rows: state of each wide row
@@ -136,16 +143,29 @@ template <int NT> __device__ __forceinline__ u32 block_excl_scan(u32 v, u32* ws,
     return r;
 }
 
-// Orders the rows by floor(log2(length)), longest first (one block).
-__global__ void __launch_bounds__(1024) k_batch_order(BatchArgs b) {
-    grid_dep_wait();
-    grid_dep_release();
+__device__ __forceinline__ u64 row_len(const BatchArgs& b, u32 i) {
+    return b.row_keys ? b.row_n[i] : b.row_off[i + 1] - b.row_off[i];
+}
+
+// Orders `rows` rows (src, or all of them) by floor(log2(length)), longest first
+// (one block), and, for the general path (`lists`), lists the wide ones.
+template <int NT>
+__device__ void order_rows(const BatchArgs& b, const u32* src, u32 rows, bool lists) {
     __shared__ u32 hist[66], start[66];
     for (u32 i = threadIdx.x; i < 66; i += blockDim.x) hist[i] = 0;
     __syncthreads();
-    for (u32 i = threadIdx.x; i < b.rows; i += blockDim.x) {
-        const u64 len = b.row_keys ? b.row_n[i] : b.row_off[i + 1] - b.row_off[i];
-        atomicAdd(&hist[len ? 64 - __clzll((long long)len) : 0], 1u);
+    constexpr int U = 4; // rows whose loads are in flight together
+    for (u32 i0 = threadIdx.x; i0 < rows; i0 += U * blockDim.x) {
+        u32 cls[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const u32 i = i0 + u * blockDim.x;
+            const u64 len = i < rows ? row_len(b, src ? src[i] : i) : 0;
+            cls[u] = i >= rows ? 66u : len ? 64 - __clzll((long long)len) : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (cls[u] < 66) atomicAdd(&hist[cls[u]], 1u);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -154,15 +174,23 @@ __global__ void __launch_bounds__(1024) k_batch_order(BatchArgs b) {
             start[k] = run;
             run += hist[k];
         }
-        *b.queue = 0;
+        b.words[2] = rows;
     }
     __syncthreads();
-    for (u32 i = threadIdx.x; i < b.rows; i += blockDim.x) {
-        const u64 len = b.row_keys ? b.row_n[i] : b.row_off[i + 1] - b.row_off[i];
-        const u32 pos = atomicAdd(&start[len ? 64 - __clzll((long long)len) : 0], 1u);
-        b.order[pos] = i;
+    for (u32 i0 = threadIdx.x; i0 < rows; i0 += U * blockDim.x) {
+        u32 cls[U], row[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const u32 i = i0 + u * blockDim.x;
+            row[u] = i < rows ? (src ? src[i] : i) : 0;
+            const u64 len = i < rows ? row_len(b, row[u]) : 0;
+            cls[u] = i >= rows ? 66u : len ? 64 - __clzll((long long)len) : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (cls[u] < 66) b.order[atomicAdd(&start[cls[u]], 1u)] = row[u];
     }
-    if (b.split == WIDE_NONE || b.row_keys != nullptr) return;
+    if (!lists || b.split == WIDE_NONE || b.row_keys != nullptr) return;
     // the wide rows in queue order, with the prefix of their tile counts
     __syncthreads();
     __shared__ u32 ws[32], tot;
@@ -175,10 +203,10 @@ __global__ void __launch_bounds__(1024) k_batch_order(BatchArgs b) {
     }
     __syncthreads();
     const unsigned char* base = static_cast<const unsigned char*>(b.keys);
-    for (u32 c0 = 0; c0 < b.rows; c0 += 1024) {
+    for (u32 c0 = 0; c0 < rows; c0 += NT) {
         const u32 i = c0 + threadIdx.x;
         u32 row = 0, flag = 0, tiles = 0;
-        if (i < b.rows) {
+        if (i < rows) {
             row = b.order[i];
             const u64 len = b.row_off[row + 1] - b.row_off[row];
             if (is_wide(b, len)) {
@@ -186,9 +214,9 @@ __global__ void __launch_bounds__(1024) k_batch_order(BatchArgs b) {
                 tiles = (u32)wide_tiles(base + b.row_off[row] * (u64)b.key_bytes, len, b.key_bytes);
             }
         }
-        const u32 rpos = block_excl_scan<1024>(flag, ws, &tot);
+        const u32 rpos = block_excl_scan<NT>(flag, ws, &tot);
         const u32 nr = tot;
-        const u32 tpos = block_excl_scan<1024>(tiles, ws, &tot);
+        const u32 tpos = block_excl_scan<NT>(tiles, ws, &tot);
         const u32 nt = tot;
         if (flag) {
             const u64 j = carry_rows + rpos;
@@ -208,6 +236,12 @@ __global__ void __launch_bounds__(1024) k_batch_order(BatchArgs b) {
         b.words[0] = (u32)carry_rows;
         b.tile_pre[carry_rows] = carry_tiles;
     }
+}
+
+__global__ void __launch_bounds__(1024) k_batch_order(BatchArgs b) {
+    grid_dep_wait();
+    grid_dep_release();
+    order_rows<1024>(b, nullptr, b.rows, b.rest == nullptr);
 }
 
 // Arguments of row `row` (keys at r0, n keys, rank k) for the selection
@@ -240,6 +274,305 @@ template <int KW> __device__ __forceinline__ typename Comp<KW>::key_t* pool_keys
 template <int KW> __device__ __forceinline__ u32* pool_idx(const BatchArgs& b, u64 off) {
     return reinterpret_cast<u32*>(b.pool + ((b.pool_pairs * sizeof(typename Comp<KW>::key_t) + 255) & ~(u64)255)) +
            off;
+}
+
+// ---------------------------------------------------- rows in one read
+// Rows of small k (k_rows), one block per row, rows longest first from a queue.
+// A row of at most CAP keys is gathered whole; a longer one is sampled (about
+// one key in 128), the sample element of rank k|S|/n + Delta is the bound, and
+// the row is streamed once, every element up to the bound going to a list in
+// shared memory; the element of rank k is selected in the list and the elements
+// up to it are written.  A list that fills up is cut back to its k smallest,
+// which tightens the bound; a row whose list ends with fewer than k elements
+// (a bound that was too low) goes to the general path, as do rows of larger k.
+//
+// One read of the keys and no candidate buffers in memory.  Bound by the latency
+// of the sampling and the selections, which the SM's other blocks cover with
+// their reads: three blocks of 256 threads to an SM (80 registers) took 308 us
+// for a program's pass over 4096 rows of 2^U(10, 18) f32 keys, four (64
+// registers, spilled) 344, two 360, two of 512 threads 376.  By levels, whose wide
+// rows went through memory three times and whose blocks waited on barriers, the
+// same pass took 912 us (68 us of each are the program's own).
+constexpr int ROWS_NT = 256;
+constexpr u32 ROWS_DRAW = 128;  // keys per draw of the sample
+constexpr int ROWS_PER_SM = 3; // resident blocks (registers and shared memory)
+constexpr u64 ROWS_MAX = 1ull << 19; // longest row: beyond, one block's read takes longer than the general path
+template <int KW> struct RowsCfg {
+    static constexpr u32 CAP = KW == 32 ? 4096 : 2048; // elements of the list (32 KB)
+    static constexpr u32 KMAX = CAP / 2;               // largest k: cutting back frees half the list
+};
+
+template <int KW> struct RowsSmem {
+    typename Comp<KW>::t list[RowsCfg<KW>::CAP];
+    HistSelSmem<KW> hs;
+    u32 n, full_at, full, row, out;
+    u32 lead[2][ROWS_NT / 32];
+    long long rank;
+};
+
+// Rank `r` among list[0..count), whatever their range.
+template <int KW>
+__device__ __noinline__ typename Comp<KW>::t rows_select(RowsSmem<KW>& sm, u32 count, u32 r) {
+    typedef typename Comp<KW>::t ct;
+    u32 mn = 0xFFFFFFFFu, mx = 0;
+    for (u32 i = threadIdx.x; i < count; i += ROWS_NT) {
+        const u32 w = (u32)(sm.list[i] >> KW);
+        mn = min(mn, w);
+        mx = max(mx, w);
+    }
+    mn = __reduce_min_sync(0xffffffffu, mn);
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if (lane_id() == 0) {
+        sm.lead[0][threadIdx.x >> 5] = mn;
+        sm.lead[1][threadIdx.x >> 5] = mx;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < ROWS_NT / 32; ++w) {
+        mn = min(mn, sm.lead[0][w]);
+        mx = max(mx, sm.lead[1][w]);
+    }
+    return block_select_hist<KW, ROWS_NT>(sm.list, count, (ct)mn << KW, ((ct)mx << KW) | (((ct)1 << KW) - 1), r, sm.hs);
+}
+
+// Keeps list[0..have)'s elements up to `thr` and opens the list again.
+template <int KW> __device__ __noinline__ void rows_cut(RowsSmem<KW>& sm, u32 have, typename Comp<KW>::t thr) {
+    typedef typename Comp<KW>::t ct;
+    constexpr u32 OWN = RowsCfg<KW>::CAP / ROWS_NT;
+    ct keep[OWN];
+    u32 km = 0;
+#pragma unroll
+    for (u32 u = 0; u < OWN; ++u) {
+        const u32 i = u * ROWS_NT + threadIdx.x;
+        keep[u] = i < have ? sm.list[i] : ~(ct)0;
+        km |= (u32)(i < have && keep[u] <= thr) << u;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        sm.n = 0;
+        sm.full = 0;
+        sm.full_at = 0xFFFFFFFFu;
+    }
+    __syncthreads();
+    u32 slot = warp_reserve((u32)__popc(km), &sm.n);
+#pragma unroll
+    for (u32 u = 0; u < OWN; ++u)
+        if ((km >> u) & 1u) sm.list[slot++] = keep[u];
+    __syncthreads();
+}
+
+template <int DT> __global__ void __launch_bounds__(ROWS_NT, ROWS_PER_SM) k_rows(BatchArgs b) {
+    grid_dep_wait();
+    typedef Key<DT> K;
+    typedef typename K::raw_t raw_t;
+    typedef typename K::key_t key_t;
+    constexpr int KW = K::KW;
+    typedef Comp<KW> C;
+    typedef typename C::t ct;
+    constexpr u32 CAP = RowsCfg<KW>::CAP, KMAX = RowsCfg<KW>::KMAX;
+    constexpr int EPV = InputSrc<DT>::EPV, NV = InputSrc<DT>::NV;
+    constexpr u32 SUB = 512; // keys of a warp's step: 16 per lane
+    constexpr u32 WARPS = ROWS_NT / 32;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    auto& sm = *reinterpret_cast<RowsSmem<KW>*>(smem_raw);
+    const u32 tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
+    const bool by_ptr = b.row_keys != nullptr;
+    auto next_row = [&]() -> u32 {
+        if (!b.ordered) return 0xFFFFFFFFu;
+        const u32 idx = atomicAdd(b.queue, 1u);
+        return idx < b.rows ? b.order[idx] : 0xFFFFFFFFu;
+    };
+    u32 ahead = !b.ordered ? blockIdx.x : tid == 0 ? next_row() : 0u; // (no more blocks than rows)
+    while (true) {
+        if (tid == 0) {
+            sm.row = ahead;
+            sm.n = 0;
+            sm.out = 0;
+            sm.full = 0;
+            sm.full_at = 0xFFFFFFFFu;
+        }
+        __syncthreads();
+        const u32 row = sm.row;
+        if (row == 0xFFFFFFFFu) break;
+        if (tid == 0) ahead = next_row(); // (needed a whole row later)
+        const u64 r0 = by_ptr ? 0 : b.row_off[row];
+        const u64 n64 = by_ptr ? b.row_n[row] : b.row_off[row + 1] - r0;
+        const u64 k64 = b.row_k[row];
+        if (k64 == 0 || k64 > n64 || n64 > 0xFFFFFFFFull) {
+            if (tid == 0) latch(b.err, ST_EINVAL);
+            __syncthreads(); // sm.row is read by all
+            continue;
+        }
+        const bool whole = n64 <= CAP;
+        if (!whole && (n64 > ROWS_MAX || k64 > KMAX)) {
+            if (tid == 0) b.rest[atomicAdd(b.nrest, 1u)] = row;
+            __syncthreads();
+            continue;
+        }
+        const u32 n = (u32)n64, k = (u32)k64;
+        const raw_t* keys = by_ptr ? static_cast<const raw_t*>(b.row_keys[row]) : static_cast<const raw_t*>(b.keys) + r0;
+        ct thr = C::from128(key_domain_max<DT>()); // elements above it are passed over
+        if (!whole) {
+            // the bound, off a sample of about n / 128 draws, one in each of as many equal parts
+            const u32 draws = min(max((n / ROWS_DRAW + 3u) & ~3u, 512u), CAP / 2);
+            for (u32 j0 = tid * 4; j0 < draws; j0 += ROWS_NT * 4) {
+                const Philox4 r = philox4x32_10(j0, row, 0x524F5753u, 0, (u32)b.seed, (u32)(b.seed >> 32));
+                raw_t x[4];
+                u32 pos[4];
+#pragma unroll
+                for (u32 q = 0; q < 4; ++q) {
+                    const u32 lo = (u32)((u64)(j0 + q) * n / draws), hi = (u32)((u64)(j0 + q + 1) * n / draws);
+                    pos[q] = lo + __umulhi(r.v[q], hi - lo);
+                    x[q] = keys[pos[q]];
+                }
+#pragma unroll
+                for (u32 q = 0; q < 4; ++q) sm.list[j0 + q] = C::make(K::fwd(x[q]), pos[q]);
+            }
+            if (tid == 0) {
+                long long jl, jr;
+                pivot_ranks(draws, n, k, b.z, false, jl, jr);
+                sm.rank = jr;
+            }
+            __syncthreads();
+            const long long jr = sm.rank;
+            if (jr < (long long)draws) thr = rows_select<KW>(sm, draws, (u32)jr);
+            __syncthreads(); // the list is free again
+        }
+        // the stream: steps of 512 keys, warp by warp, on 16-byte boundaries
+        const u32 head = (u32)((reinterpret_cast<uintptr_t>(keys) & 15u) / sizeof(raw_t));
+        const uint4* vec = reinterpret_cast<const uint4*>(reinterpret_cast<uintptr_t>(keys) & ~(uintptr_t)15);
+        const u32 ext = n + head, subs = (ext + SUB - 1) / SUB;
+        u32 t = warp;
+        auto inside = [&](u32 s) { return s < subs && s * SUB >= head && (s + 1) * SUB <= ext; };
+        auto load = [&](u32 s, uint4(&v)[NV]) {
+            if (inside(s)) {
+#pragma unroll
+                for (int j = 0; j < NV; ++j) v[j] = __ldcs(vec + (size_t)s * (SUB / EPV) + j * 32 + lane);
+            }
+        };
+        while (true) {
+            const key_t tk = (key_t)C::key(thr);
+            const u32 tx = C::idx(thr);
+            // ties with the bound's key count up to its position
+            const RawBound<DT> upto = RawBound<DT>::le(tk), under = RawBound<DT>::le((key_t)(tk - 1));
+            uint4 v[NV];
+            load(t, v);
+            while (t < subs) {
+                uint4 w[NV];
+                load(t + WARPS, w);
+                const u32 e0 = t * SUB; // slot q is element e0 + ((q / EPV) * 32 + lane) * EPV + q % EPV
+                auto pos = [&](int q) -> u32 { return e0 + (u32)((q / EPV) * 32 + lane) * EPV + (u32)(q % EPV) - head; };
+                raw_t rr[16];
+                u32 hit = 0;
+                if (inside(t)) {
+                    InputSrc<DT>::unpack_raw(v, rr);
+                    const u32 p0 = e0 - head;
+                    if (p0 + (SUB - 1) <= tx) hit = tile_le_dispatch<DT>(rr, upto, true);
+                    else if (p0 > tx) hit = tile_le_dispatch<DT>(rr, under, tk != 0);
+                    else {
+#pragma unroll
+                        for (int q = 0; q < 16; ++q) hit |= (u32)(C::make(K::fwd(rr[q]), pos(q)) <= thr) << q;
+                    }
+                } else { // the row's first or last step
+#pragma unroll
+                    for (int q = 0; q < 16; ++q) {
+                        const u32 e = e0 + (u32)((q / EPV) * 32 + lane) * EPV + (u32)(q % EPV);
+                        rr[q] = 0;
+                        if (e >= head && e < ext) {
+                            rr[q] = reinterpret_cast<const raw_t*>(vec)[e];
+                            hit |= (u32)(C::make(K::fwd(rr[q]), e - head) <= thr) << q;
+                        }
+                    }
+                }
+                if (__any_sync(0xffffffffu, hit)) {
+                    const u32 total = __reduce_add_sync(0xffffffffu, (u32)__popc(hit));
+                    u32 at = 0;
+                    if (lane == 0) at = atomicAdd(&sm.n, total);
+                    at = __shfl_sync(0xffffffffu, at, 0);
+                    if (at + total > CAP) { // full: every later reservation fails too, so nothing lies beyond `at`
+                        if (lane == 0) {
+                            atomicMin(&sm.full_at, at);
+                            *(volatile u32*)&sm.full = 1;
+                        }
+                        break;
+                    }
+                    // one hit of every lane that has any at a time (few: one or two turns)
+                    const u32 below = lanemask_lt();
+                    u32 bal = __ballot_sync(0xffffffffu, hit);
+                    do {
+                        if (hit) {
+                            const u32 q = (u32)(__ffs(hit) - 1);
+                            hit &= hit - 1;
+                            sm.list[at + (u32)__popc(bal & below)] = C::make(K::fwd(pick16(rr, q)), pos((int)q));
+                        }
+                        at += (u32)__popc(bal);
+                        bal = __ballot_sync(0xffffffffu, hit);
+                    } while (bal);
+                }
+                t += WARPS;
+                if (__any_sync(0xffffffffu, *(volatile u32*)&sm.full)) break;
+#pragma unroll
+                for (int j = 0; j < NV; ++j) v[j] = w[j];
+            }
+            __syncthreads();
+            if (!sm.full) break;
+            // cut the list back to its k smallest and go on below the k-th
+            const u32 have = min(sm.n, sm.full_at);
+            if (have < k) break; // (k <= CAP / 2 and a step adds at most 512: cannot be)
+            thr = rows_select<KW>(sm, have, k - 1);
+            rows_cut<KW>(sm, have, thr);
+        }
+        const u32 count = min(sm.n, sm.full_at);
+        if (count < k) { // the bound was too low
+            if (tid == 0) b.rest[atomicAdd(b.nrest, 1u)] = row;
+            __syncthreads();
+            continue;
+        }
+        const ct kth = count == k && k == 1 ? sm.list[0] : rows_select<KW>(sm, count, k - 1);
+        raw_t* ok = by_ptr ? static_cast<raw_t*>(b.row_out_keys[row]) : static_cast<raw_t*>(b.out_keys) + b.out_off[row];
+        u32* oi = by_ptr ? b.row_out_idx[row] : b.out_idx + b.out_off[row];
+        for (u32 base = 0; base < count; base += ROWS_NT * 8) {
+            u32 selm = 0;
+#pragma unroll
+            for (u32 u = 0; u < 8; ++u) {
+                const u32 i = base + u * ROWS_NT + tid;
+                selm |= (u32)(i < count && sm.list[i] <= kth) << u;
+            }
+            u32 slot = warp_reserve((u32)__popc(selm), &sm.out);
+            while (selm) {
+                const u32 u = (u32)(__ffs(selm) - 1);
+                selm &= selm - 1;
+                const ct c = sm.list[base + u * ROWS_NT + tid];
+                if (slot < k) {
+                    ok[slot] = K::inv((key_t)C::key(c));
+                    oi[slot] = C::idx(c);
+                }
+                ++slot;
+            }
+        }
+        if (tid == 0) {
+            *(by_ptr ? static_cast<raw_t*>(b.row_kth_key[row]) : static_cast<raw_t*>(b.kth_keys) + row) =
+                K::inv((key_t)C::key(kth));
+            *(by_ptr ? b.row_kth_idx[row] : b.kth_idx + row) = C::idx(kth);
+        }
+        __syncthreads(); // the row's shared words are done with
+    }
+    // the last block orders the rows left to the general path
+    if (tid == 0) {
+        __threadfence();
+        sm.row = atomicAdd(b.rows_done, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!sm.row) return;
+    __threadfence();
+    const u32 left = *(volatile u32*)b.nrest;
+    __syncthreads();
+    order_rows<ROWS_NT>(b, b.rest, left, true);
+    if (tid == 0) {
+        *b.rows_done = 0;
+        *b.nrest = 0;
+        *b.queue = 0;
+    }
 }
 
 // First level of the wide rows, part 1 (one block of 256 threads per row,
@@ -576,12 +909,18 @@ __global__ void __launch_bounds__(NT, (BatchVariant<Key<DT>::KW, NT>::MINB)) k_b
     while (true) {
         if (threadIdx.x == 0) {
             const u32 idx = atomicAdd(b.queue, 1u);
-            s_row = idx < b.rows ? b.order[idx] : 0xFFFFFFFFu;
+            s_row = idx < b.words[2] ? b.order[idx] : 0xFFFFFFFFu;
         }
         __syncthreads();
         const u32 row = s_row;
         __syncthreads();
-        if (row == 0xFFFFFFFFu) break;
+        if (row == 0xFFFFFFFFu) { // the last block leaves the queue as it found it
+            if (threadIdx.x == 0 && atomicAdd(b.rows_done, 1u) == gridDim.x - 1) {
+                *b.rows_done = 0;
+                *b.queue = 0;
+            }
+            break;
+        }
         const bool by_ptr = b.row_keys != nullptr;
         const u64 r0 = by_ptr ? 0 : b.row_off[row];
         const u64 n = by_ptr ? b.row_n[row] : b.row_off[row + 1] - r0;
@@ -695,14 +1034,29 @@ template <int DT> static topk_status wide_setup(int device, int& pass_per_sm, in
 }
 
 template <int DT, int NT>
-static topk_status launch_batched(topk_ctx* ctx, const BatchArgs& b, cudaStream_t st) {
+static topk_status launch_batched(topk_ctx* ctx, BatchArgs b, cudaStream_t st) {
     constexpr int KW = Key<DT>::KW;
     topk_status rs;
     const int per_sm = batched_blocks_per_sm<DT, NT>(ctx->device, rs);
     if (rs != TOPK_OK) return rs;
     int pass_per_sm = 1, plan_per_sm = 1;
     if (b.split != WIDE_NONE && (rs = wide_setup<DT>(ctx->device, pass_per_sm, plan_per_sm)) != TOPK_OK) return rs;
-    cudaError_t e = launch_dep(k_batch_order, 1, 1024, 0, st, 1, b);
+    // rows that all start at once need no order
+    b.ordered = b.rows > (u32)ctx->sms * ROWS_PER_SM;
+    const bool order = b.ordered || !b.rest;
+    cudaError_t e = order ? launch_dep(k_batch_order, 1, 1024, 0, st, 1, b) : cudaSuccess;
+    if (e == cudaSuccess && b.rest) {
+        static std::atomic<uint64_t> attr{0};
+        const uint64_t bit = 1ull << (ctx->device & 63);
+        if (!(attr.load() & bit)) {
+            if (cudaFuncSetAttribute(k_rows<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)sizeof(RowsSmem<KW>)) != cudaSuccess)
+                return TOPK_ECUDA;
+            attr.fetch_or(bit);
+        }
+        const int grid = (int)std::min<u64>(b.rows, (u64)ctx->sms * ROWS_PER_SM);
+        e = launch_dep(k_rows<DT>, grid, ROWS_NT, sizeof(RowsSmem<KW>), st, 1, b);
+    }
     if (e == cudaSuccess && b.split != WIDE_NONE) {
         e = launch_dep(k_wide_plan<DT>, ctx->sms * plan_per_sm, WIDE_PLAN_NT, sizeof(BatchSmem<KW, WIDE_PLAN_NT>), st, 1,
                        b);
@@ -711,7 +1065,7 @@ static topk_status launch_batched(topk_ctx* ctx, const BatchArgs& b, cudaStream_
     }
     if (e == cudaSuccess) e = launch_dep(k_batched<DT, NT>, ctx->sms * per_sm, NT, sizeof(BatchSmem<KW, NT>), st, 1, b);
     if (e != cudaSuccess) return cuda_status(e);
-    count_launch(ctx, b.split != WIDE_NONE ? 4 : 2);
+    count_launch(ctx, (order ? 1 : 0) + (b.rest ? 1 : 0) + (b.split != WIDE_NONE ? 3 : 1));
     return cuda_status(cudaGetLastError());
 }
 
@@ -728,19 +1082,19 @@ template <int DT> static int batched_max_grid(topk_ctx* ctx, topk_status& rs) {
 // Scratch regions of one batched launch over `rows` rows with `grid` blocks
 // (and, with wide rows, the per-row arrays and the candidate pool).
 struct BatchCarve {
-    size_t order, queue, states, cand;
-    size_t wide, words, tile_pre, done, rstate, rcand, pool_next, pool;
+    size_t order, rest, words, states, cand;
+    size_t wide, tile_pre, done, rstate, rcand, pool_next, pool;
 };
 template <int DT> static Carve batch_carve(u32 rows, int grid, bool wide, BatchCarve& bc) {
     typedef typename Key<DT>::key_t key_t;
     Carve cv;
     bc.order = cv.take(4ull * rows);
-    bc.queue = cv.take(256);
+    bc.rest = cv.take(4ull * rows);
+    bc.words = cv.take(256);
     bc.states = cv.take(sizeof(SelState) * (size_t)grid);
     bc.cand = cv.take((size_t)grid * 2 * BATCH_CAP * (sizeof(key_t) + 4));
     if (wide) {
         bc.wide = cv.take(4ull * rows);
-        bc.words = cv.take(256);
         bc.tile_pre = cv.take(8ull * (rows + 1));
         bc.done = cv.take(4ull * rows);
         bc.rstate = cv.take(sizeof(SelState) * (size_t)rows);
@@ -752,7 +1106,7 @@ template <int DT> static Carve batch_carve(u32 rows, int grid, bool wide, BatchC
 }
 
 template <int DT>
-static topk_status run_batched(topk_ctx* ctx, BatchArgs b, int threads, cudaStream_t st) {
+static topk_status run_batched(topk_ctx* ctx, BatchArgs b, int threads, bool by_rows, cudaStream_t st) {
     typedef typename Key<DT>::key_t key_t;
     constexpr int KW = Key<DT>::KW;
     topk_status rs = TOPK_OK;
@@ -772,12 +1126,15 @@ static topk_status run_batched(topk_ctx* ctx, BatchArgs b, int threads, cudaStre
     if (rs != TOPK_OK) return rs;
     char* base = static_cast<char*>(ctx->scratch.base);
     b.order = reinterpret_cast<u32*>(base + bc.order);
-    b.queue = reinterpret_cast<u32*>(base + bc.queue);
+    b.words = reinterpret_cast<u32*>(base + bc.words);
+    b.queue = ctx->d_counter + 4;
+    b.nrest = ctx->d_counter + 5;
+    b.rows_done = ctx->d_counter + 6;
+    b.rest = by_rows ? reinterpret_cast<u32*>(base + bc.rest) : nullptr;
     b.states = reinterpret_cast<SelState*>(base + bc.states);
     b.cand = base + bc.cand;
     if (wide) {
         b.wide = reinterpret_cast<u32*>(base + bc.wide);
-        b.words = reinterpret_cast<u32*>(base + bc.words);
         b.tile_pre = reinterpret_cast<u64*>(base + bc.tile_pre);
         b.done = reinterpret_cast<u32*>(base + bc.done);
         b.rstate = reinterpret_cast<SelState*>(base + bc.rstate);
@@ -791,14 +1148,15 @@ static topk_status run_batched(topk_ctx* ctx, BatchArgs b, int threads, cudaStre
     return launch_batched<DT, 1024>(ctx, b, st);
 }
 
-static topk_status run_batched_dt(topk_ctx* ctx, topk_dtype dtype, const BatchArgs& b, int threads,
+// `by_rows`: rows of small k in one read (k_rows) before the general path.
+static topk_status run_batched_dt(topk_ctx* ctx, topk_dtype dtype, const BatchArgs& b, int threads, bool by_rows,
                                   cudaStream_t st) {
     switch (dtype) {
-    case TOPK_U32: return run_batched<DT_U32>(ctx, b, threads, st);
-    case TOPK_I32: return run_batched<DT_I32>(ctx, b, threads, st);
-    case TOPK_F32: return run_batched<DT_F32>(ctx, b, threads, st);
-    case TOPK_BF16: return run_batched<DT_BF16>(ctx, b, threads, st);
-    case TOPK_U64: return run_batched<DT_U64>(ctx, b, threads, st);
+    case TOPK_U32: return run_batched<DT_U32>(ctx, b, threads, by_rows, st);
+    case TOPK_I32: return run_batched<DT_I32>(ctx, b, threads, by_rows, st);
+    case TOPK_F32: return run_batched<DT_F32>(ctx, b, threads, by_rows, st);
+    case TOPK_BF16: return run_batched<DT_BF16>(ctx, b, threads, by_rows, st);
+    case TOPK_U64: return run_batched<DT_U64>(ctx, b, threads, by_rows, st);
     default: return TOPK_EINVAL;
     }
 }
@@ -835,7 +1193,7 @@ topk_status batched_by_pointers(topk_ctx* ctx, topk_dtype dtype, u32 rows, const
         b.sample = it->second.sample_size;
         b.finish_T = it->second.finish_threshold;
     }
-    return run_batched_dt(ctx, dtype, b, threads, st);
+    return run_batched_dt(ctx, dtype, b, threads, true, st);
 }
 
 static int log2_floor(u64 v) { return v ? 63 - __builtin_clzll(v) : 0; }
@@ -917,6 +1275,9 @@ extern "C" topk_status topk_select_batched(topk_ctx* ctx, const void* d_keys, co
     if (cudaSetDevice(ctx->device) != cudaSuccess) return TOPK_ECUDA;
     topk_params p{};
     if (params) p = *params;
+    // settings given by the caller are the general path's
+    const bool general = p.block_threads || p.sample_size || p.finish_threshold || p.split_rows ||
+                         (p.flags & (TOPK_FLAG_RAW_DELTA | TOPK_FLAG_TINY_CAND));
     if (p.block_threads == 0 && p.sample_size == 0 && p.finish_threshold == 0 && p.split_rows == 0) {
         auto it = ctx->tuned.find({(int)dtype, log2_floor(rows)});
         if (it != ctx->tuned.end()) {
@@ -930,7 +1291,7 @@ extern "C" topk_status topk_select_batched(topk_ctx* ctx, const void* d_keys, co
     const BatchArgs b = batch_args(ctx, d_keys, d_row_off, d_row_k, rows, dtype, d_out_keys, d_out_idx, d_out_off,
                                    d_kth_keys, d_kth_idx, p, threads);
     ctx->last_kind = LAST_BATCHED;
-    return run_batched_dt(ctx, dtype, b, threads, static_cast<cudaStream_t>(stream));
+    return run_batched_dt(ctx, dtype, b, threads, !general, static_cast<cudaStream_t>(stream));
 }
 
 extern "C" topk_status topk_tune_batched(topk_ctx* ctx, const void* d_keys, const uint64_t* d_row_off,
@@ -971,7 +1332,7 @@ extern "C" topk_status topk_tune_batched(topk_ctx* ctx, const void* d_keys, cons
                 float ms = 0.f;
                 for (int rep = 0; rep < 4 && rs == TOPK_OK; ++rep) { // one warm-up, best of three
                     if (cudaEventRecord(e0, st) != cudaSuccess) rs = TOPK_ECUDA;
-                    if (rs == TOPK_OK) rs = run_batched_dt(ctx, dtype, b, nt, st);
+                    if (rs == TOPK_OK) rs = run_batched_dt(ctx, dtype, b, nt, true, st);
                     if (rs == TOPK_OK && cudaEventRecord(e1, st) != cudaSuccess) rs = TOPK_ECUDA;
                     if (rs == TOPK_OK && cudaEventSynchronize(e1) != cudaSuccess) rs = TOPK_ECUDA;
                     float t = 0.f;
@@ -1002,7 +1363,7 @@ extern "C" topk_status topk_tune_batched(topk_ctx* ctx, const void* d_keys, cons
             float ms = 0.f;
             for (int rep = 0; rep < 4 && rs == TOPK_OK; ++rep) {
                 if (cudaEventRecord(e0, st) != cudaSuccess) rs = TOPK_ECUDA;
-                if (rs == TOPK_OK) rs = run_batched_dt(ctx, dtype, b, nt, st);
+                if (rs == TOPK_OK) rs = run_batched_dt(ctx, dtype, b, nt, true, st);
                 if (rs == TOPK_OK && cudaEventRecord(e1, st) != cudaSuccess) rs = TOPK_ECUDA;
                 if (rs == TOPK_OK && cudaEventSynchronize(e1) != cudaSuccess) rs = TOPK_ECUDA;
                 float t = 0.f;
@@ -1027,7 +1388,7 @@ extern "C" topk_status topk_tune_batched(topk_ctx* ctx, const void* d_keys, cons
     const BatchArgs b = batch_args(ctx, d_keys, d_row_off, d_row_k, rows, dtype, d_out_keys, d_out_idx, d_out_off,
                                    d_kth_keys, d_kth_idx, choice, nt);
     ctx->last_kind = LAST_BATCHED;
-    rs = run_batched_dt(ctx, dtype, b, nt, st);
+    rs = run_batched_dt(ctx, dtype, b, nt, true, st);
     return rs == TOPK_OK ? topk_status_sync(ctx, stream) : rs;
 }
 
