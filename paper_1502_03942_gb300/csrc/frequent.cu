@@ -270,9 +270,9 @@ __global__ void __launch_bounds__(FQ_NT, 3) k_freq_count(FreqArgs a) {
 // the candidates sit in a shared-memory hash table of words
 // (candidate number << 32 | object); every block counts its part and adds its counts to exact[] at
 // the end.  The candidates are the most frequent objects, so many threads
-// hit the same few counters: MODE 0 (k* <= FQ_PT_MAX) gives every thread
-// its own counters (plain increments), MODE 1 (k* <= FQ_PW_MAX) every warp
-// (shared-memory atomics within the warp only), MODE 2 one set per block.
+// hit the same few counters: up to FQ_PT_MAX candidates every thread has its
+// own (k_freq_exact_few), up to FQ_PW_MAX every warp (MODE 1: shared-memory
+// atomics within the warp only), above that one set per block (MODE 2).
 constexpr u32 FQ_PT_MAX = 32;
 constexpr int FQ_XQUADS = 4; // 4-object groups per thread per iteration (loads in flight)
 constexpr u32 FQ_PW_MAX = 1024;
@@ -287,7 +287,7 @@ struct ExactArgs {
 };
 
 __host__ __device__ inline size_t fq_exact_counters(int mode, u32 kstar) {
-    return mode == 0 ? (size_t)kstar * FQ_NT : mode == 1 ? (size_t)kstar * (FQ_NT / 32) : (size_t)kstar;
+    return mode == 1 ? (size_t)kstar * (FQ_NT / 32) : (size_t)kstar;
 }
 
 // Position of an object in the recount's candidate table: one
@@ -297,7 +297,6 @@ __device__ __forceinline__ u32 fq_cand_pos(u32 v, u32 log_slots) { return (v * 0
 
 // Counts one object: a table word is (candidate number << 32) | object, an
 // empty slot has a negative candidate number.
-template <int MODE>
 __device__ __forceinline__ void fq_recount_one(const u64* slot, u32 log_slots, u32* my, u32 v) {
     const u32 mask = (1u << log_slots) - 1;
     u32 h = fq_cand_pos(v, log_slots);
@@ -310,9 +309,113 @@ __device__ __forceinline__ void fq_recount_one(const u64* slot, u32 log_slots, u
             c = (int)(w >> 32);
         } while (c >= 0 && (u32)w != v);
     }
-    if (c >= 0) {
-        if (MODE == 0) my[(u32)c * FQ_NT] += 1;
-        else atomicAdd(&my[c], 1u);
+    if (c >= 0) atomicAdd(&my[c], 1u);
+}
+
+// The recount of at most FQ_PT_MAX candidates (they are the most frequent
+// objects: about 28% of a Zipf input).  Bound by shared-memory accesses: a
+// probe of one hash table by 32 lanes takes about six cycles of bank conflicts
+// for 8-byte slots, and a quarter of the lanes probe twice.  So a multiplier is
+// searched that gives the candidates different slots (no probing), and every
+// lane has its own copy of the slots' objects (slot s of lane l at s * 32 + l: no
+// conflicts); a match finds the candidate's number in a byte table and counts in
+// the thread's own counter.  On 2^28 Zipf objects, 32 candidates: 186 us,
+// 290 us with one probed table.
+constexpr u32 FQ_SLOTS = 256;      // slots of the lanes' tables
+constexpr u32 FQ_TRIES = 4096;     // multipliers tried (about one in eight separates 32 candidates)
+struct FqFew {
+    u32 key[FQ_SLOTS * 32];
+    u32 cnt[FQ_PT_MAX * FQ_NT];
+    unsigned char num[FQ_SLOTS];
+    u32 tried;                     // first multiplier that separates the candidates
+};
+__device__ __forceinline__ u32 fq_multiplier(u32 t) { return (0x2545F491u + t * 0x9E3779B8u) | 0x80000001u; }
+__device__ __forceinline__ u32 fq_few_slot(u32 v, u32 mul) { return (v * mul) >> 24; }
+static_assert(FQ_SLOTS == 256, "a slot is the product's top byte");
+
+template <bool VEC> __global__ void __launch_bounds__(FQ_NT, 2) k_freq_exact_few(ExactArgs a) {
+    extern __shared__ __align__(16) unsigned char fq_smem[];
+    FqFew& L = *reinterpret_cast<FqFew*>(fq_smem);
+    const u32 tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (u32 c = tid; c < FQ_PT_MAX * FQ_NT; c += FQ_NT) L.cnt[c] = 0;
+    if (tid == 0) L.tried = FQ_TRIES;
+    grid_dep_wait(); // the candidates come from the previous selection
+    __syncthreads();
+    const u32 cand = lane < a.kstar ? (u32)a.cand[lane] : 0u;
+    for (u32 t = warp; t < FQ_TRIES; t += FQ_NT / 32) {
+        if (*(volatile u32*)&L.tried <= t) break;
+        // lanes without a candidate get a value of their own
+        const u32 s = lane < a.kstar ? fq_few_slot(cand, fq_multiplier(t)) : FQ_SLOTS + lane;
+        const u32 alike = __match_any_sync(0xffffffffu, s);
+        if (__all_sync(0xffffffffu, (alike & (alike - 1)) == 0)) {
+            if (lane == 0) atomicMin(&L.tried, t);
+            break;
+        }
+    }
+    __syncthreads();
+    const u32 t0 = L.tried;
+    const bool apart = t0 < FQ_TRIES; // else every object is compared with every candidate
+    const u32 mul = fq_multiplier(t0);
+    // a free slot holds an object of another slot: 0 lies in slot 0, 1 in slot mul >> 24 (at least 128)
+    for (u32 i = tid; i < FQ_SLOTS * 32; i += FQ_NT) L.key[i] = i < 32 ? 1u : 0u;
+    __syncthreads();
+    for (u32 c = warp; c < a.kstar; c += FQ_NT / 32) {
+        const u32 o = (u32)a.cand[c], s = apart ? fq_few_slot(o, mul) : c;
+        L.key[s * 32 + lane] = o;
+        if (lane == 0) L.num[s] = (unsigned char)c;
+    }
+    __syncthreads();
+    auto count1 = [&](u32 v) {
+        if (apart) {
+            const u32 s = fq_few_slot(v, mul);
+            if (L.key[s * 32 + lane] == v) L.cnt[(u32)L.num[s] * FQ_NT + tid] += 1;
+        } else {
+            u32 c = 0;
+            while (c < a.kstar && L.key[c * 32 + lane] != v) ++c;
+            if (c < a.kstar) L.cnt[c * FQ_NT + tid] += 1;
+        }
+    };
+    auto count4 = [&](const uint4& x) {
+        if (!apart) {
+#pragma unroll 1
+            for (int e = 0; e < 4; ++e) count1(u4at(x, e));
+            return;
+        }
+        u32 s[4], k[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            s[e] = fq_few_slot(u4at(x, e), mul);
+            k[e] = L.key[s[e] * 32 + lane];
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            if (k[e] == u4at(x, e)) L.cnt[(u32)L.num[s[e]] * FQ_NT + tid] += 1;
+    };
+    const u64 quads = (a.n + 3) / 4;
+    const u64 tile_quads = (u64)FQ_NT * FQ_XQUADS;
+    const u64 full_tiles = VEC ? (a.n / 4) / tile_quads : 0;
+    for (u64 t = blockIdx.x; t * tile_quads < quads; t += gridDim.x) {
+        const u64 q0 = t * tile_quads + tid;
+        if (VEC && t < full_tiles) {
+            uint4 x[FQ_XQUADS];
+#pragma unroll
+            for (int j = 0; j < FQ_XQUADS; ++j) x[j] = ld_stream(reinterpret_cast<const uint4*>(a.obj) + q0 + j * FQ_NT);
+#pragma unroll
+            for (int j = 0; j < FQ_XQUADS; ++j) count4(x[j]);
+        } else {
+            for (int j = 0; j < FQ_XQUADS; ++j) {
+                const u64 i0 = (q0 + (u64)j * FQ_NT) * 4;
+                for (int e = 0; e < 4; ++e)
+                    if (i0 + e < a.n) count1(__ldcs(a.obj + i0 + e));
+            }
+        }
+    }
+    __syncthreads();
+    for (u32 c = warp; c < a.kstar; c += FQ_NT / 32) {
+        u32 sum = 0;
+        for (u32 t = lane; t < FQ_NT; t += 32) sum += L.cnt[c * FQ_NT + t];
+        sum = __reduce_add_sync(0xffffffffu, sum);
+        if (lane == 0 && sum) atomicAdd(&a.exact[c], sum);
     }
 }
 
@@ -335,8 +438,8 @@ __global__ void __launch_bounds__(FQ_NT, 3) k_freq_exact(ExactArgs a) {
             h = (h + 1) & (slots - 1);
     }
     __syncthreads();
-    // this thread's (MODE 0) or warp's (MODE 1) counters
-    u32* my = MODE == 0 ? cnt + threadIdx.x : MODE == 1 ? cnt + (threadIdx.x >> 5) * a.kstar : cnt;
+    u32* my = MODE == 1 ? cnt + (threadIdx.x >> 5) * a.kstar : cnt; // this warp's counters
+
     const u64 quads = (a.n + 3) / 4;
     const u64 tile_quads = (u64)FQ_NT * FQ_XQUADS;
     const u64 full_tiles = VEC ? (a.n / 4) / tile_quads : 0;
@@ -348,16 +451,16 @@ __global__ void __launch_bounds__(FQ_NT, 3) k_freq_exact(ExactArgs a) {
             for (int j = 0; j < FQ_XQUADS; ++j) x[j] = ld_stream(reinterpret_cast<const uint4*>(a.obj) + q0 + j * FQ_NT);
 #pragma unroll
             for (int j = 0; j < FQ_XQUADS; ++j) {
-                fq_recount_one<MODE>(slot, a.log_slots, my, x[j].x);
-                fq_recount_one<MODE>(slot, a.log_slots, my, x[j].y);
-                fq_recount_one<MODE>(slot, a.log_slots, my, x[j].z);
-                fq_recount_one<MODE>(slot, a.log_slots, my, x[j].w);
+                fq_recount_one(slot, a.log_slots, my, x[j].x);
+                fq_recount_one(slot, a.log_slots, my, x[j].y);
+                fq_recount_one(slot, a.log_slots, my, x[j].z);
+                fq_recount_one(slot, a.log_slots, my, x[j].w);
             }
         } else {
             for (int j = 0; j < FQ_XQUADS; ++j) {
                 const u64 i0 = (q0 + (u64)j * FQ_NT) * 4;
                 for (int e = 0; e < 4; ++e)
-                    if (i0 + e < a.n) fq_recount_one<MODE>(slot, a.log_slots, my, __ldcs(a.obj + i0 + e));
+                    if (i0 + e < a.n) fq_recount_one(slot, a.log_slots, my, __ldcs(a.obj + i0 + e));
             }
         }
     }
@@ -369,10 +472,9 @@ __global__ void __launch_bounds__(FQ_NT, 3) k_freq_exact(ExactArgs a) {
     }
     // sum the private counters of each candidate: one warp per candidate
     const u32 lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const u32 copies = MODE == 0 ? FQ_NT : FQ_NT / 32;
     for (u32 c = warp; c < a.kstar; c += FQ_NT / 32) {
         u32 sum = 0;
-        for (u32 t = lane; t < copies; t += 32) sum += MODE == 0 ? cnt[c * FQ_NT + t] : cnt[t * a.kstar + c];
+        for (u32 t = lane; t < FQ_NT / 32; t += 32) sum += cnt[t * a.kstar + c];
         for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
         if (lane == 0 && sum) atomicAdd(&a.exact[c], sum);
     }
@@ -592,8 +694,9 @@ topk_status topk_frequent(topk_ctx* ctx, const void* d_objects, uint64_t n, topk
     x.log_slots = fq_exact_log_slots(kstar);
     x.exact = exact;
     const int mode = kstar <= FQ_PT_MAX ? 0 : kstar <= FQ_PW_MAX ? 1 : 2;
-    const size_t smem = (size_t)(1u << x.log_slots) * 8 + 4 * fq_exact_counters(mode, kstar);
-    void (*exact_kernels[3][2])(ExactArgs) = {{k_freq_exact<0, false>, k_freq_exact<0, true>},
+    const size_t smem =
+        mode == 0 ? sizeof(FqFew) : (size_t)(1u << x.log_slots) * 8 + 4 * fq_exact_counters(mode, kstar);
+    void (*exact_kernels[3][2])(ExactArgs) = {{k_freq_exact_few<false>, k_freq_exact_few<true>},
                                               {k_freq_exact<1, false>, k_freq_exact<1, true>},
                                               {k_freq_exact<2, false>, k_freq_exact<2, true>}};
     auto ek = exact_kernels[mode][vec ? 1 : 0];
@@ -602,7 +705,8 @@ topk_status topk_frequent(topk_ctx* ctx, const void* d_objects, uint64_t n, topk
     if (!(attr_mask.load() & bit)) {
         for (int m = 0; m < 3; ++m) {
             const u32 kmax = m == 0 ? FQ_PT_MAX : m == 1 ? FQ_PW_MAX : FQ_EXACT_MAX;
-            const int max_smem = (int)((1u << fq_exact_log_slots(kmax)) * 8 + 4 * fq_exact_counters(m, kmax));
+            const int max_smem = m == 0 ? (int)sizeof(FqFew)
+                                        : (int)((1u << fq_exact_log_slots(kmax)) * 8 + 4 * fq_exact_counters(m, kmax));
             for (int v = 0; v < 2; ++v)
                 if (cudaFuncSetAttribute(exact_kernels[m][v], cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          max_smem) != cudaSuccess)
