@@ -186,24 +186,42 @@ def _torch():
     return torch
 
 
+_codes = None
+
+
 def dtype_code(t) -> int:
-    torch = _torch()
-    m = {torch.uint32: TOPK_U32, torch.int32: TOPK_I32, torch.float32: TOPK_F32,
-         torch.bfloat16: TOPK_BF16, torch.uint64: TOPK_U64}
-    if t.dtype not in m:
+    global _codes
+    if _codes is None:
+        torch = _torch()
+        _codes = {torch.uint32: TOPK_U32, torch.int32: TOPK_I32, torch.float32: TOPK_F32,
+                  torch.bfloat16: TOPK_BF16, torch.uint64: TOPK_U64}
+    code = _codes.get(t.dtype)
+    if code is None:
         raise TypeError(f"unsupported key dtype {t.dtype}")
-    return m[t.dtype]
+    return code
+
+
+# Marshalling takes most of a small selection's time on the host: the current
+# stream's handle is asked for without building a Stream object (2.8 us of a
+# 9 us call), addresses go to ctypes as plain integers (declared void*), and the
+# dtype table is built once.
+_raw_stream = None
 
 
 def _stream_ptr(stream):
+    """The cudaStream_t of ``stream``, or of the current device's current stream."""
+    global _raw_stream
+    if stream is not None:
+        return stream.cuda_stream
     torch = _torch()
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    if _raw_stream is None:
+        _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or \
+            (lambda device: torch.cuda.current_stream(device).cuda_stream)
+    return _raw_stream(torch.cuda.current_device())
 
 
 def _ptr(t):
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 TOPK_SPLIT_NONE = 0xFFFFFFFF
