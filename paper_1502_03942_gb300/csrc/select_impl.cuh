@@ -204,11 +204,11 @@ constexpr int TMA_CONS = 256;
 constexpr int TMA_NT = TMA_CONS + 32;
 constexpr u64 WAIT_LIMIT_NS = 200ull * 1000 * 1000;
 
-// Ring geometry.  A sparse or counting pass has 2 blocks per SM (the warps'
-// buffers and the bins take 40 KB of a block); with three smaller blocks and
-// buffers of half the size the counting pass is slower (322 us against 286 for
-// the median of 2^28 f32 keys), because every tile is then appended in two
-// parts.  A dense pass holds two stages per block (one counted, one being written
+// Ring geometry.  A sparse pass has 2 blocks per SM, with room for a whole
+// tile's hits in every warp's buffer; a counting pass, which has more to do for
+// every key, 3 blocks with smaller rings and buffers (median of 2^28 f32 keys 275
+// us against 282 with the sparse pass's geometry; k = 1024 of them 199 against
+// 194).  A dense pass holds two stages per block (one counted, one being written
 // out), with 3 blocks (24 consumer warps) per SM, 2 for 64-bit keys.
 enum : int { PM_SPARSE = 0, PM_DENSE = 1, PM_COUNT = 2 }; // what a first-level pass does with a (few; many; counted)
 template <int DT, int MODE = PM_SPARSE> struct TmaCfg {
@@ -216,9 +216,10 @@ template <int DT, int MODE = PM_SPARSE> struct TmaCfg {
     static constexpr u32 W = sizeof(typename Key<DT>::raw_t);
     static constexpr u32 TILE = TMA_CONS * 16; // elements per stage
     static constexpr u32 BYTES = TILE * W;     // 8, 16 or 32 KiB
-    static constexpr u32 STAGES = W == 2 ? 8 : W == 4 ? 4 : 3; // two blocks (dense: three) fit an SM
+    static constexpr u32 STAGES = MODE == PM_COUNT ? (W == 2 ? 6 : 3) : (W == 2 ? 8 : W == 4 ? 4 : 3);
+    static constexpr u32 WB_CAP = W == 8 || MODE == PM_COUNT ? 256 : 512; // entries of a warp's buffer
     static constexpr u32 SMEM = STAGES * BYTES;
-    static constexpr int MIN_BLOCKS = DENSE ? (W == 8 ? 2 : 3) : 1;
+    static constexpr int MIN_BLOCKS = MODE == PM_SPARSE ? 1 : W == 8 ? (DENSE ? 2 : 1) : 3;
 };
 
 // Raw key bits of this thread's 16 slots from a stage (slot q at vector
@@ -235,13 +236,14 @@ __device__ __forceinline__ void load_raw_stage(const unsigned char* stage, typen
 // A warp's buffer of elements on their way out of a first-level pass, packed:
 // a tile's hits take consecutive slots (one shared-memory atomic per lane that has
 // any), so a flush writes whole rows of 32.  One flush in about 30 tiles waits
-// for its reservation, which the other warps and the ring cover.  (Per-lane
-// queues, whose rows are as long as the fullest lane's, and which classified every
-// entry again, took 0.27 ms for the counting pass on 2^28 f32 keys at k = n / 2,
-// 0.33 ms with the bins kept; packed: 0.235 ms with the bins.)
-template <int KW> struct WarpBuf {
-    static constexpr u32 CAP = KW == 32 ? 512 : 256; // a tile's 512 hits, or half of them
-    typename Comp<KW>::key_t k[CAP];
+// for its reservation, which the other warps and the ring cover.  Entries keep
+// the raw key bits; the rows of a flush turn them into images.  (Per-lane queues,
+// whose rows are as long as the fullest lane's, and which classified every entry
+// again, took 0.33 ms for the counting pass on 2^28 f32 keys at k = n / 2, packed
+// 0.235 ms, and 0.18 ms with the masks built off the integer pipe.)
+template <int KW, u32 N> struct WarpBuf {
+    static constexpr u32 CAP = N;
+    typename Comp<KW>::key_t k[CAP]; // raw key bits
     u32 i[CAP];
     u32 n;
 };
@@ -249,15 +251,17 @@ template <int KW> struct WarpBuf {
 // Writes a warp's `cnt` entries (all at most pr): those below pl to the output,
 // unless the buffer holds b elements only (ONLY_B), the rest to the
 // candidates and their bins.
-template <int DT, bool ONLY_B>
-__device__ __forceinline__ void wb_flush(WarpBuf<Key<DT>::KW>& w, u32 cnt, typename Comp<Key<DT>::KW>::t pl,
+template <int DT, bool ONLY_B, class WB>
+__device__ __forceinline__ void wb_flush(WB& w, u32 cnt, typename Comp<Key<DT>::KW>::t pl,
                                          const Sink<DT>& sink, const BinHist<Key<DT>::KW>& bins) {
+    typedef Key<DT> K;
+    typedef typename K::raw_t raw_t;
     typedef Comp<Key<DT>::KW> C;
     const u32 lane = lane_id(), below = lanemask_lt();
     __syncwarp();
     u32 ca = 0;
     if constexpr (!ONLY_B) {
-        for (u32 j = lane; j < cnt; j += 32) ca += (u32)(C::make(w.k[j], w.i[j]) < pl);
+        for (u32 j = lane; j < cnt; j += 32) ca += (u32)(C::make(K::fwd((raw_t)w.k[j]), w.i[j]) < pl);
         ca = __reduce_add_sync(0xffffffffu, ca);
     }
     u64 ra = 0, rb = 0;
@@ -271,7 +275,7 @@ __device__ __forceinline__ void wb_flush(WarpBuf<Key<DT>::KW>& w, u32 cnt, typen
     for (u32 j0 = 0; j0 < cnt; j0 += 32) {
         const u32 j = j0 + lane;
         const bool in = j < cnt;
-        const auto kv = in ? w.k[j] : (typename C::key_t)0;
+        const typename C::key_t kv = in ? K::fwd((raw_t)w.k[j]) : (typename C::key_t)0;
         const u32 iv = in ? w.i[j] : 0u;
         if constexpr (ONLY_B) {
             if (in) {
@@ -293,36 +297,42 @@ __device__ __forceinline__ void wb_flush(WarpBuf<Key<DT>::KW>& w, u32 cnt, typen
     __syncwarp();
 }
 
-// Appends the slots of `hit` (key_at(q), pos(q) for a lane-dependent q); `cnt` is
-// the number of entries, the same in every lane.  All 32 lanes call.
-template <int DT, bool ONLY_B, class PosF, class KeyAt>
-__device__ __forceinline__ void wb_append(WarpBuf<Key<DT>::KW>& w, u32& cnt, u32 hit, PosF pos, KeyAt key_at,
-                                          typename Comp<Key<DT>::KW>::t pl, const Sink<DT>& sink,
+// Appends the slots of `hit`: slot q's key bits are raw_at(off) and its position
+// is first + off, off = off_of(q) (q and off differ by lane).  `cnt` is the number
+// of entries, the same in every lane.  All 32 lanes call.
+template <int DT, bool ONLY_B, class WB, class OffOf, class RawAt>
+__device__ __forceinline__ void wb_append(WB& w, u32& cnt, u32 hit, u32 first, OffOf off_of,
+                                          RawAt raw_at, typename Comp<Key<DT>::KW>::t pl, const Sink<DT>& sink,
                                           const BinHist<Key<DT>::KW>& bins) {
-    constexpr u32 CAP = WarpBuf<Key<DT>::KW>::CAP;
-    constexpr u32 PARTS = 512 / CAP; // slots taken at once: as many as always fit
-    if (!__any_sync(0xffffffffu, hit)) return;
-    const u32 all = hit;
-#pragma unroll 1
-    for (u32 h = 0; h < PARTS; ++h) {
-        u32 m = PARTS == 1 ? all : (all >> (h * (16 / PARTS)) << (h * (16 / PARTS))) & ((1u << ((h + 1) * (16 / PARTS))) - 1u);
-        const u32 mine = (u32)__popc(m);
-        const u32 total = __reduce_add_sync(0xffffffffu, mine);
-        if (cnt + total > CAP) {
+    constexpr u32 CAP = WB::CAP;
+    const u32 total = __reduce_add_sync(0xffffffffu, (u32)__popc(hit));
+    if (total == 0) return;
+    auto add = [&](u32 m, u32 n) {
+        if (cnt + n > CAP) {
             wb_flush<DT, ONLY_B>(w, cnt, pl, sink, bins);
             cnt = 0;
         }
         if (m) {
-            u32 slot = atomicAdd(&w.n, mine);
+            u32 slot = atomicAdd(&w.n, (u32)__popc(m));
             do {
-                const u32 q = (u32)(__ffs(m) - 1);
+                const u32 off = off_of((u32)(__ffs(m) - 1));
                 m &= m - 1;
-                w.k[slot] = key_at(q);
-                w.i[slot] = pos((int)q);
+                w.k[slot] = raw_at(off);
+                w.i[slot] = first + off;
                 ++slot;
             } while (m);
         }
-        cnt += total;
+        cnt += n;
+    };
+    if (total <= CAP) {
+        add(hit, total);
+    } else { // nearly the whole tile: as many slots at a time as always fit
+        constexpr u32 S = CAP / 32;
+#pragma unroll 1
+        for (u32 h = 0; h < 16; h += S) {
+            const u32 m = (hit >> h) & ((1u << S) - 1u);
+            add(m << h, __reduce_add_sync(0xffffffffu, (u32)__popc(m)));
+        }
     }
 }
 
@@ -331,18 +341,19 @@ __device__ __forceinline__ void wb_append(WarpBuf<Key<DT>::KW>& w, u32& cnt, u32
 // rank-k pair alone).  A tile that holds neither pivot's position is tested
 // with one comparison of raw key bits per element and pivot (tile bounds), the
 // rare other tile on the pair; the few hits go through the warp's buffer.  No
-// block barrier.  On 2^28 f32 keys at k = n / 2 the counting pass takes 0.235
+// block barrier.  On 2^28 f32 keys at k = n / 2 the counting pass takes 0.18
 // ms, against 0.47 ms for the pass that writes a.
 template <int DT, bool COUNT>
 __device__ void tma_consume_few(const SelArgs& a, const SelState& s, const unsigned char* stages, uint64_t* full,
-                                uint64_t* empty, u64 my_n, u32* dead, WarpBuf<Key<DT>::KW>& wb,
+                                uint64_t* empty, u64 my_n, u32* dead,
+                                WarpBuf<Key<DT>::KW, TmaCfg<DT, COUNT ? PM_COUNT : PM_SPARSE>::WB_CAP>& wb,
                                 const BinHist<Key<DT>::KW>& bins) {
     typedef Key<DT> K;
     typedef typename K::raw_t raw_t;
     typedef typename K::key_t key_t;
     typedef Comp<K::KW> C;
     typedef typename C::t ct;
-    typedef TmaCfg<DT> Cfg;
+    typedef TmaCfg<DT, COUNT ? PM_COUNT : PM_SPARSE> Cfg;
     constexpr u32 EPV = InputSrc<DT>::EPV;
     const Sink<DT> sink = make_sink<DT>(a, s);
     const ct pl = C::from128(s.pl), pr = C::from128(s.pr);
@@ -351,7 +362,8 @@ __device__ void tma_consume_few(const SelArgs& a, const SelState& s, const unsig
     if (lane == 0) wb.n = 0;
     __syncwarp();
     const TileBounds<DT> tbd = TileBounds<DT>::make(pl, pr);
-    u64 na = 0;
+    u32 na = 0; // (a lane sees fewer than 2^32 keys)
+    const u32 one = hidden_one();
     u32 cnt = 0, stg = 0, parity = 0;
     for (u64 i = 0; i < my_n; ++i) {
         bool ok = !*(volatile u32*)dead;
@@ -366,30 +378,31 @@ __device__ void tma_consume_few(const SelArgs& a, const SelState& s, const unsig
         const u32 tb = (u32)((blockIdx.x + i * gridDim.x) * (u64)Cfg::TILE);
         const u32 ib = tb + threadIdx.x * EPV;
         auto pos = [&](int q) -> u32 { return ib + (u32)(q / (int)EPV) * (TMA_CONS * EPV) + (u32)(q % (int)EPV); };
-        u32 ma = 0, le = 0;
+        u32 hit = 0;
         if (ok) {
             raw_t rr[16];
             load_raw_stage<DT>(stages + (size_t)stg * Cfg::BYTES, rr);
             RawBound<DT> ba, bb;
             bool any_a, any_l;
-            if (tbd.get(tb, tb + Cfg::TILE - 1, ba, bb, any_a, any_l)) {
-                if constexpr (COUNT) tile_masks_dispatch<DT>(rr, ba, bb, any_a, any_l, ma, le);
-                else le = tile_le_dispatch<DT>(rr, bb, any_l);
+            const bool away = tbd.get(tb, tb + Cfg::TILE - 1, ba, bb, any_a, any_l);
+            if (COUNT ? away && any_a && any_l : away) {
+                if constexpr (COUNT) tile_count_dispatch<DT>(rr, ba, bb, one, na, hit);
+                else hit = tile_le_dispatch<DT>(rr, bb, any_l);
             } else {
 #pragma unroll
                 for (int q = 0; q < 16; ++q) {
                     const ct c = C::make(K::fwd(rr[q]), pos(q));
-                    if (COUNT) ma |= (u32)(c < pl) << q;
-                    le |= (u32)(c <= pr) << q;
+                    const bool in_a = COUNT && c < pl;
+                    na += (u32)in_a;
+                    hit |= (u32)(!in_a && c <= pr) << q;
                 }
             }
         }
-        if (COUNT) na += (u32)__popc(ma);
         // the hits' keys come from the stage, which is released after them
         const unsigned char* mine = stages + (size_t)stg * Cfg::BYTES + threadIdx.x * 16u;
-        wb_append<DT, COUNT>(wb, cnt, le & ~ma, pos, [&](u32 sq) {
-            return K::fwd(*reinterpret_cast<const raw_t*>(mine + (sq / EPV) * (TMA_CONS * 16u) + (sq % EPV) * sizeof(raw_t)));
-        }, pl, sink, bins);
+        wb_append<DT, COUNT>(wb, cnt, hit, ib, [](u32 q) { return (q / EPV) * (TMA_CONS * EPV) + q % EPV; },
+                             [&](u32 off) { return *reinterpret_cast<const raw_t*>(mine + off * sizeof(raw_t)); }, pl,
+                             sink, bins);
         __syncwarp();
         if (ok && lane == 0) mbar_arrive(&empty[stg]); // the stage may be refilled
         if (++stg == Cfg::STAGES) {
@@ -414,12 +427,15 @@ __device__ void tma_consume_few(const SelArgs& a, const SelState& s, const unsig
         }
         ma &= valid;
         na += (u32)__popc(ma);
-        wb_append<DT, COUNT>(wb, cnt, le & valid & ~ma, pos, [&](u32 sq) { return pick16(kk, sq); }, pl, sink, bins);
+        wb_append<DT, COUNT>(wb, cnt, le & valid & ~ma, (u32)tb + threadIdx.x * EPV,
+                             [](u32 q) { return (q / EPV) * (TMA_CONS * EPV) + q % EPV; },
+                             [&](u32 off) { return static_cast<const raw_t*>(a.keys)[tb + threadIdx.x * EPV + off]; }, pl,
+                             sink, bins);
     }
     if (cnt) wb_flush<DT, COUNT>(wb, cnt, pl, sink, bins);
     if constexpr (COUNT) {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) na += __shfl_xor_sync(0xffffffffu, (unsigned long long)na, o);
+        for (int o = 16; o > 0; o >>= 1) na += __shfl_xor_sync(0xffffffffu, na, o); // (of fewer than 2^32 in all)
         if (lane == 0 && na) atomicAdd((unsigned long long*)sink.cnt_a, (unsigned long long)na);
     }
 }
@@ -635,7 +651,7 @@ __global__ void __launch_bounds__(TMA_NT, (TmaCfg<DT, MODE>::MIN_BLOCKS)) k_pass
     __shared__ __align__(8) uint64_t full[Cfg::STAGES];
     __shared__ __align__(8) uint64_t empty[Cfg::STAGES];
     __shared__ PassSmem<TMA_CONS> ps;
-    __shared__ __align__(16) unsigned char wb_raw[DENSE ? 16 : sizeof(WarpBuf<KW>) * (TMA_CONS / 32)];
+    __shared__ __align__(16) unsigned char wb_raw[DENSE ? 16 : sizeof(WarpBuf<KW, Cfg::WB_CAP>) * (TMA_CONS / 32)];
     __shared__ DenseSmem ds;
     __shared__ u32 hist[HB_BINS];
     __shared__ EpilogueSmem es;
@@ -689,7 +705,7 @@ __global__ void __launch_bounds__(TMA_NT, (TmaCfg<DT, MODE>::MIN_BLOCKS)) k_pass
         return;
     }
     const BinHist<KW> bins = make_bins<DT>(a, hist);
-    WarpBuf<KW>* wb = reinterpret_cast<WarpBuf<KW>*>(wb_raw) + (DENSE ? 0 : threadIdx.x >> 5);
+    auto* wb = reinterpret_cast<WarpBuf<KW, Cfg::WB_CAP>*>(wb_raw) + (DENSE ? 0 : threadIdx.x >> 5);
     if constexpr (!DENSE) tma_consume_few<DT, MODE == PM_COUNT>(a, s, stages, full, empty, my_n, &dead, *wb, bins);
     else tma_consume_dense<DT>(a, s, stages, full, empty, my_n, &dead, ds, ps, bins);
     grid_dep_release(); // this block's stream has ended: the next kernel may start taking its place
