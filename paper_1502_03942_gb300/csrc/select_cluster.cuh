@@ -316,10 +316,15 @@ template <int KW> struct PlanSmem {
 // j mod 4); the sample elements of ranks k|S|/n -/+ Delta are selected over the
 // cluster.  Also clears the bins of the pass that follows.
 //
+// `first` = 0: pivots among the candidates that the passes so far have left, when
+// they are more than the finish holds (they sit on a few distant values, so that
+// equal bins resolved nothing); returns at once otherwise, and where the window
+// was narrowed on its source (every draw has to count).
+//
 // Replaces a sampling kernel and a one-block pivot kernel that passed the
 // sample through global memory: 17 us on 2^28 f32 keys, 12 us now
 // (30 us and 16 us where most of the sample ties with the pivots).
-template <int DT> __global__ void __launch_bounds__(CL_NT) k_plan(SelArgs a) {
+template <int DT> __global__ void __launch_bounds__(CL_NT) k_plan(SelArgs a, int first) {
     cl_arrive(); // (no remote access before every block of the cluster has started)
     grid_dep_wait();
     grid_dep_release();
@@ -332,23 +337,31 @@ template <int DT> __global__ void __launch_bounds__(CL_NT) k_plan(SelArgs a) {
     constexpr u32 DPT = Lim<KW>::ELEMS / (CL_BLOCKS * CL_NT); // draws per thread
     static_assert(DPT >= 1 && DPT <= 4 && 4 % DPT == 0, "a thread's draws lie in one Philox block");
     const u32 gid = cl_rank() * CL_NT + threadIdx.x;
-    const u32 m = (u32)a.n, draws = a.sample;
+    const SelState* g = a.st;
+    if (!first && (g->phase != PH_RUN || g->src == SRC_INPUT || g->m_win != g->m_src ||
+                   g->m_src <= (u64)CL_BLOCKS * Lim<KW>::ELEMS))
+        return;
+    const u32 m = first ? (u32)a.n : (u32)g->m_src, draws = a.sample;
+    const u64 k = first ? a.k : g->k_rem;
+    const u32 level = first ? 0u : g->level, src_id = first ? (u32)SRC_INPUT : g->src;
     cl_clear(sel);
     // (independent of the draws, whose loads it covers)
     long long jl, jr;
-    pivot_ranks(draws, a.n, a.k, a.z, (a.flags & TOPK_FLAG_RAW_DELTA) != 0, jl, jr);
+    pivot_ranks(draws, m, k, a.z, (a.flags & TOPK_FLAG_RAW_DELTA) != 0, jl, jr);
     const long long top = (long long)draws - 1;
     const u32 r1 = (u32)(jr < 0 ? 0 : jr > top ? top : jr);
     const u32 r0 = jl < 0 ? r1 : (u32)(jl > top ? top : jl); // (an unused lower rank follows the upper one)
-    if (a.bins)
+    if (first && a.bins)
         for (u32 i = gid; i < HB_BINS; i += CL_BLOCKS * CL_NT) a.bins->h[i] = 0;
     ct c[DPT];
     const InputSrc<DT> src = InputSrc<DT>::make(a.keys, m);
+    const CandSrc<KW> csrc{static_cast<const typename K::key_t*>(a.cand_key[src_id == SRC_CAND1 ? 1 : 0]),
+                           a.cand_idx[src_id == SRC_CAND1 ? 1 : 0], m};
     {
         const u32 p = a.parts < m ? a.parts : m;
         const u32 len = m / p, rem = m - len * p;
         const u32 j0 = gid * DPT;
-        const Philox4 r = philox4x32_10(j0 & ~3u, 0, 0x53414D50u, 0, (u32)a.seed, (u32)(a.seed >> 32));
+        const Philox4 r = philox4x32_10(j0 & ~3u, level, 0x53414D50u, 0, (u32)a.seed, (u32)(a.seed >> 32));
 #pragma unroll
         for (u32 q = 0; q < DPT; ++q) {
             const u32 j = j0 + q;
@@ -360,7 +373,10 @@ template <int DT> __global__ void __launch_bounds__(CL_NT) k_plan(SelArgs a) {
             const u32 pos = plo + (u32)(((u64)rv * psz) >> 32);
             typename K::key_t kq = 0;
             u32 x = 0;
-            if (j < draws) src.at(pos, kq, x);
+            if (j < draws) {
+                if (first) src.at(pos, kq, x);
+                else csrc.at(pos, kq, x);
+            }
             c[q] = C::make(kq, x);
         }
     }
@@ -386,6 +402,20 @@ template <int DT> __global__ void __launch_bounds__(CL_NT) k_plan(SelArgs a) {
             if (q < mine) f(c[q]);
     }, wlo, whi, rk, total);
     if (gid != 0) return;
+    if (!first) { // arms the next pass over the candidates
+        SelState* w = a.st;
+        if (!ok) return; // (left to the finish)
+        w->pl = jl >= 0 ? (u128)sel.res[0] : w->lo;
+        w->pr = jr <= top ? (u128)sel.res[1] : w->hi;
+        w->dst = src_id == SRC_CAND0 ? SRC_CAND1 : SRC_CAND0;
+        w->cnt_a = 0;
+        w->cnt_b = 0;
+        w->dense = jl >= 0 && (jl + 1) * 16 > (long long)draws ? 1u : 0u;
+        w->level = level + 1;
+        w->levels_grid++;
+        w->pending = 1;
+        return;
+    }
     SelState s = initial_state<DT>(a);
     const ct hi = C::from128(s.hi);
     const ct pl = jl >= 0 ? sel.res[0] : (ct)0, pr = jr <= top ? sel.res[1] : hi;

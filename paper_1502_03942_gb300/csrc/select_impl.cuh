@@ -11,6 +11,8 @@
 //                        second pass between the ends of rank k's bin
 //   k_pass   (grid)      that second pass, over the candidates (usually a few
 //                        thousand are left); returns at once when not armed
+//   k_plan, k_pass       once more, when many candidates are expected: a level by
+//                        sampling for candidates that the bins did not part
 //   k_finish (1 cluster) selection of rank k among what is left, the rest of
 //                        the output and the rank-k pair
 // Inputs of at most T keys take k_finish alone.
@@ -748,8 +750,10 @@ __device__ typename Comp<KW>::t block_extreme(typename Comp<KW>::t v, bool want_
     return out;
 }
 
-template <int DT>
-__global__ void __launch_bounds__(EXT_NT) k_extreme(SelArgs a, int want_max, u32* counter, void* partials_v) {
+// MAX: k = n; COPY: it copies every pair out (not for the rank-k pair alone).
+template <int DT, bool MAX, bool COPY>
+__global__ void __launch_bounds__(EXT_NT) k_extreme(SelArgs a, u32* counter, void* partials_v) {
+    constexpr bool want_max = MAX, copy = COPY;
     grid_dep_wait();
     grid_dep_release();
     typedef Key<DT> K;
@@ -761,7 +765,6 @@ __global__ void __launch_bounds__(EXT_NT) k_extreme(SelArgs a, int want_max, u32
     __shared__ u32 is_last;
     ct* partials = static_cast<ct*>(partials_v);
     const InputSrc<DT> src = InputSrc<DT>::make(a.keys, a.n);
-    const bool copy = want_max != 0 && !a.kth_only; // k = n also copies every pair out
     raw_t* ok_out = static_cast<raw_t*>(a.out_keys);
     ct best = want_max ? (ct)0 : C::max_value();
     constexpr u64 TILE = (u64)EXT_NT * 16;
@@ -951,8 +954,10 @@ static topk_status enqueue_select(topk_ctx* ctx, SelArgs a, const Tuning& tu, in
     const u64 n = a.n, k = a.k;
     if (k == 1 || k == n) {
         if (ctx) profile_pass_begin(ctx, st);
-        const cudaError_t e = launch_dep(k_extreme<DT>, sms * EXT_BLOCKS_PER_SM, EXT_NT, 0, st, 1, a,
-                                         k == n && n > 1 ? 1 : 0, counter, partials);
+        const auto kern = !(k == n && n > 1) ? k_extreme<DT, false, false>
+                          : a.kth_only       ? k_extreme<DT, true, false>
+                                             : k_extreme<DT, true, true>;
+        const cudaError_t e = launch_dep(kern, sms * EXT_BLOCKS_PER_SM, EXT_NT, 0, st, 1, a, counter, partials);
         if (e != cudaSuccess) return cuda_status(e);
         if (ctx) {
             profile_pass_end(ctx, st);
@@ -978,6 +983,13 @@ static topk_status enqueue_select(topk_ctx* ctx, SelArgs a, const Tuning& tu, in
                           TmaCfg<DT, PM_SPARSE>::SMEM, st, 1, a);
     };
     const bool one = n <= tu.T;
+    // Candidates on a few distant values (ties of integer-valued floats, say) fall
+    // into a few bins, and what the second pass then leaves would be streamed by
+    // the finish's eight blocks, at about 40 us for 4e6 of them and every step: from
+    // 2^20 expected candidates on, one more level by sampling stands ready
+    // (1.3 us for each of its two kernels when it is not needed; 2^28 f32 Zipf keys at
+    // k = n / 2 take 578 us with it and 733 without).
+    const bool resample = !one && est_bracket(n, k, tu.sample, tu.z) >= 1048576.0;
     cudaError_t e = cudaSuccess;
     if (!one) {
         // (the finish holds CL_BLOCKS times as many, but a second pass over more
@@ -986,19 +998,23 @@ static topk_status enqueue_select(topk_ctx* ctx, SelArgs a, const Tuning& tu, in
         // the bins are kept where they are likely to be needed
         if (1.2 * est_bracket(n, k, tu.sample, tu.z) <= (double)a.list_max && !(tu.flags & TOPK_FLAG_RAW_DELTA))
             a.bins = nullptr;
-        e = launch_dep(k_plan<DT>, CL_BLOCKS, CL_NT, sizeof(PlanSmem<KW>), st, CL_BLOCKS, a);
+        e = launch_dep(k_plan<DT>, CL_BLOCKS, CL_NT, sizeof(PlanSmem<KW>), st, CL_BLOCKS, a, 1);
         if (e != cudaSuccess) return cuda_status(e);
         if (ctx) profile_pass_begin(ctx, st);
         e = first_pass();
         if (e != cudaSuccess) return cuda_status(e);
         if (ctx) profile_pass_end(ctx, st);
         e = launch_dep(k_pass<DT>, pass_grid<DT>(sms, false), PASS_NT, 0, st, 1, a);
+        if (e == cudaSuccess && resample) {
+            e = launch_dep(k_plan<DT>, CL_BLOCKS, CL_NT, sizeof(PlanSmem<KW>), st, CL_BLOCKS, a, 0);
+            if (e == cudaSuccess) e = launch_dep(k_pass<DT>, pass_grid<DT>(sms, false), PASS_NT, 0, st, 1, a);
+        }
         if (e != cudaSuccess) return cuda_status(e);
     }
     const int fin = one && n <= FIN_SOLO ? 1 : CL_BLOCKS; // (the kernel leaves a short source to one block)
     e = launch_dep(k_finish<DT>, fin, CL_NT, sizeof(FinSmem<KW>), st, fin, a, one ? 1 : 0);
     if (e != cudaSuccess) return cuda_status(e);
-    if (ctx) count_launch(ctx, one ? 1 : 4);
+    if (ctx) count_launch(ctx, one ? 1 : resample ? 6 : 4);
     return cuda_status(cudaGetLastError());
 }
 
