@@ -81,8 +81,9 @@ typedef struct {
     uint32_t partitions;       /* p: sampling partitions (the paper's PEs) */
     uint32_t sample_size;      /* s: sample drawn per recursion level */
     uint32_t buckets;          /* reserved; the method uses 3 (a, b, c) */
-    uint32_t finish_threshold; /* T: at most this many candidates are
-                                  finished by one thread block */
+    uint32_t finish_threshold; /* T: inputs of at most this many keys are
+                                  selected by one launch; batched: at most this
+                                  many candidates are finished by one block */
     float delta_factor;        /* z: pivot margin in standard deviations */
     uint32_t flags;            /* TOPK_FLAG_* */
     uint32_t block_threads;    /* topk_select_batched: threads per block
@@ -260,10 +261,13 @@ topk_status topk_runs_delete_min_flexible(topk_ctx *ctx, const void *d_keys,
  * (a fixed pool of 2^23 candidate pairs; a row it cannot hold is selected
  * by one block).
  * When params is NULL, or leaves block_threads, sample_size,
- * finish_threshold and split_rows all zero, the choice remembered by
- * topk_tune_batched for this dtype and row count (power-of-two bucket) is
- * used if there is one, else 1024 threads, a 2048-element sample, the
- * largest T and a split length of 2^15. */
+ * finish_threshold and split_rows all zero, rows of at most 2^19 keys whose k is
+ * at most 2048 (1024 for u64), and rows of at most 4096 (2048) keys, are read
+ * once by one block each and selected from a list in shared memory; for the
+ * others the choice remembered by topk_tune_batched for this dtype and row count
+ * (power-of-two bucket) is used if there is one, else 1024 threads, a
+ * 2048-element sample, the largest T and a split length of 2^15.  Settings that
+ * a call gives itself apply to all its rows. */
 topk_status topk_select_batched(topk_ctx *ctx, const void *d_keys,
                                 const uint64_t *d_row_off, const uint32_t *d_row_k,
                                 uint32_t rows, topk_dtype dtype, void *d_out_keys,

@@ -1,7 +1,6 @@
 // select_block.cuh — one thread block runs whole recursion levels of the
 // selection: planning (sample + pivots), a block-wide pass, the branch, and
-// the final exact selection among at most T candidates.  Used by the
-// single-selection finish (select_impl.cuh: k_finish) and by the batched
+// the final exact selection among at most T candidates.  Used by the batched
 // kernels (batched.cu), where every block selects whole rows.
 #pragma once
 
@@ -309,18 +308,9 @@ __device__ __forceinline__ void block_level(const SelArgs& a, SM& sm) {
     __syncthreads();
 }
 
-// The same, out of line: its register demand then does not weigh on a
-// caller that seldom needs it.
-template <int DT, bool ONLY_EXACT, class SM>
-__device__ __noinline__ void block_level_outlined(const SelArgs& a, SM& sm) {
-    block_level<DT, ONLY_EXACT>(a, sm);
-}
-
 // Recursion levels run by this block alone until at most T elements remain in
 // the source, then the exact finish.  Precondition: no pass pending.
-// OUTLINED keeps the level code out of line (for callers whose source is
-// usually at most T already).
-template <int DT, bool ONLY_EXACT, bool OUTLINED = false, class SM>
+template <int DT, bool ONLY_EXACT, class SM>
 __device__ void block_levels_and_finish(const SelArgs& a, SM& sm) {
     SelState* g = a.st;
     for (u32 it = 0; it < MAX_BLOCK_LEVELS; ++it) {
@@ -328,8 +318,7 @@ __device__ void block_levels_and_finish(const SelArgs& a, SM& sm) {
             block_finish<DT>(a, sm);
             return;
         }
-        if (OUTLINED) block_level_outlined<DT, ONLY_EXACT>(a, sm);
-        else block_level<DT, ONLY_EXACT>(a, sm);
+        block_level<DT, ONLY_EXACT>(a, sm);
     }
     if (threadIdx.x == 0) {
         g->status = ST_EINTERNAL;
