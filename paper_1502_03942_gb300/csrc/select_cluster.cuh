@@ -325,15 +325,19 @@ template <int KW> struct PlanSmem {
 // sample through global memory: 17 us on 2^28 f32 keys, 12 us now
 // (30 us and 16 us where most of the sample ties with the pivots).
 template <int DT> __global__ void __launch_bounds__(CL_NT) k_plan(SelArgs a, int first) {
-    cl_arrive(); // (no remote access before every block of the cluster has started)
-    grid_dep_wait();
-    grid_dep_release();
     typedef Key<DT> K;
     constexpr int KW = K::KW;
     typedef Comp<KW> C;
     typedef typename C::t ct;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     auto& sel = reinterpret_cast<PlanSmem<KW>*>(smem_raw)->sel;
+    // The barrier before the first remote access, in two halves: it also has to
+    // cover the clearing, since a block that cleared late would wipe out what
+    // another has already reduced into it.
+    cl_clear(sel);
+    cl_arrive();
+    grid_dep_wait();
+    grid_dep_release();
     constexpr u32 DPT = Lim<KW>::ELEMS / (CL_BLOCKS * CL_NT); // draws per thread
     static_assert(DPT >= 1 && DPT <= 4 && 4 % DPT == 0, "a thread's draws lie in one Philox block");
     const u32 gid = cl_rank() * CL_NT + threadIdx.x;
@@ -344,7 +348,6 @@ template <int DT> __global__ void __launch_bounds__(CL_NT) k_plan(SelArgs a, int
     const u32 m = first ? (u32)a.n : (u32)g->m_src, draws = a.sample;
     const u64 k = first ? a.k : g->k_rem;
     const u32 level = first ? 0u : g->level, src_id = first ? (u32)SRC_INPUT : g->src;
-    cl_clear(sel);
     // (independent of the draws, whose loads it covers)
     long long jl, jr;
     pivot_ranks(draws, m, k, a.z, (a.flags & TOPK_FLAG_RAW_DELTA) != 0, jl, jr);
@@ -401,6 +404,7 @@ template <int DT> __global__ void __launch_bounds__(CL_NT) k_plan(SelArgs a, int
         for (u32 q = 0; q < DPT; ++q)
             if (q < mine) f(c[q]);
     }, wlo, whi, rk, total);
+    if (!ok) cl_sync(); // (the same in every block) no block leaves while others read its bins
     if (gid != 0) return;
     if (!first) { // arms the next pass over the candidates
         SelState* w = a.st;
