@@ -306,6 +306,7 @@ template <int KW> struct RowsSmem {
     typename Comp<KW>::t list[RowsCfg<KW>::CAP];
     HistSelSmem<KW> hs;
     u32 n, full_at, full, row, out;
+    u32 last; // the block is the kernel's last (a word of its own: `row` may still be read)
     u32 lead[2][ROWS_NT / 32];
     long long rank;
 };
@@ -560,10 +561,10 @@ template <int DT> __global__ void __launch_bounds__(ROWS_NT, ROWS_PER_SM) k_rows
     // the last block orders the rows left to the general path
     if (tid == 0) {
         __threadfence();
-        sm.row = atomicAdd(b.rows_done, 1u) == gridDim.x - 1;
+        sm.last = atomicAdd(b.rows_done, 1u) == gridDim.x - 1;
     }
     __syncthreads();
-    if (!sm.row) return;
+    if (!sm.last) return;
     __threadfence();
     const u32 left = *(volatile u32*)b.nrest;
     __syncthreads();

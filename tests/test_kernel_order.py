@@ -37,6 +37,16 @@ def test_plan_clears_before_the_cluster_barrier():
     assert 0 <= after.find("if (!ok) cl_sync();") < after.index("return")
 
 
+def test_rows_queue_word_is_written_at_the_top_only():
+    """k_rows: the word that hands out a row is read by every thread after the
+    loop's barrier, the last time without another barrier behind it, so it is
+    written at the top of the loop and nowhere else."""
+    body = body_of("batched.cu", "k_rows")
+    writes = [m.start() for m in re.finditer(r"\bsm\.row\s*=(?!=)", body)]
+    loop = body.index("while (true)")
+    assert len(writes) == 1 and loop < writes[0] < body.index("__syncthreads()", loop)
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("n,k", [(20000, 7000), (1 << 21, 1 << 20)])
 def test_plan_repeats(n, k):
