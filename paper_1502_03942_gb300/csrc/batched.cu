@@ -1315,6 +1315,8 @@ extern "C" topk_status topk_tune_batched(topk_ctx* ctx, const void* d_keys, cons
         cudaEventDestroy(e0);
         return TOPK_ECUDA;
     }
+    // (every row by the general path, whose settings these are: a call that gives
+    // them runs all its rows there, and rows left by k_rows run there too)
     topk_status rs = TOPK_OK;
     topk_params choice = b0;
     float best_ms = 0.f;
@@ -1333,7 +1335,7 @@ extern "C" topk_status topk_tune_batched(topk_ctx* ctx, const void* d_keys, cons
                 float ms = 0.f;
                 for (int rep = 0; rep < 4 && rs == TOPK_OK; ++rep) { // one warm-up, best of three
                     if (cudaEventRecord(e0, st) != cudaSuccess) rs = TOPK_ECUDA;
-                    if (rs == TOPK_OK) rs = run_batched_dt(ctx, dtype, b, nt, true, st);
+                    if (rs == TOPK_OK) rs = run_batched_dt(ctx, dtype, b, nt, false, st);
                     if (rs == TOPK_OK && cudaEventRecord(e1, st) != cudaSuccess) rs = TOPK_ECUDA;
                     if (rs == TOPK_OK && cudaEventSynchronize(e1) != cudaSuccess) rs = TOPK_ECUDA;
                     float t = 0.f;
@@ -1364,7 +1366,7 @@ extern "C" topk_status topk_tune_batched(topk_ctx* ctx, const void* d_keys, cons
             float ms = 0.f;
             for (int rep = 0; rep < 4 && rs == TOPK_OK; ++rep) {
                 if (cudaEventRecord(e0, st) != cudaSuccess) rs = TOPK_ECUDA;
-                if (rs == TOPK_OK) rs = run_batched_dt(ctx, dtype, b, nt, true, st);
+                if (rs == TOPK_OK) rs = run_batched_dt(ctx, dtype, b, nt, false, st);
                 if (rs == TOPK_OK && cudaEventRecord(e1, st) != cudaSuccess) rs = TOPK_ECUDA;
                 if (rs == TOPK_OK && cudaEventSynchronize(e1) != cudaSuccess) rs = TOPK_ECUDA;
                 float t = 0.f;
@@ -1389,7 +1391,7 @@ extern "C" topk_status topk_tune_batched(topk_ctx* ctx, const void* d_keys, cons
     const BatchArgs b = batch_args(ctx, d_keys, d_row_off, d_row_k, rows, dtype, d_out_keys, d_out_idx, d_out_off,
                                    d_kth_keys, d_kth_idx, choice, nt);
     ctx->last_kind = LAST_BATCHED;
-    rs = run_batched_dt(ctx, dtype, b, nt, true, st);
+    rs = run_batched_dt(ctx, dtype, b, nt, false, st);
     return rs == TOPK_OK ? topk_status_sync(ctx, stream) : rs;
 }
 
