@@ -40,16 +40,24 @@ __device__ __forceinline__ u64 atomic_read(u64* p) {
     return atomicAdd(reinterpret_cast<unsigned long long*>(p), 0ull);
 }
 
+// What the finish's list holds: what is left undecided above this is planned and
+// passed over once more.
+template <int KW> constexpr u64 FIN_LIST = (u64)CL_BLOCKS * Lim<KW>::ELEMS;
+
 // The branch of Algorithm "select", taken by the last block of a pass once
 // every block's counts are in (block-done counter; nobody waits), and, after a
-// first level that leaves more candidates than the finish holds, the pivots of a
-// second pass: the ends of the bin that holds rank k (exact counts, so that pass
-// cannot miss).  All NT threads call, after the block's own atomics.
+// first level that leaves more candidates than the finish takes at once, the pivots
+// of a second pass: the ends of the bin that holds rank k (exact counts, so that
+// pass cannot miss).  The bins also serve when there were more candidates than the
+// buffer holds; the pass then reads the input again.  Where neither is
+// possible the second pass plans for itself (plan_here).
+// `planned`: the state of a pass that did so.  All NT threads call, after the
+// block's own atomics.
 struct EpilogueSmem {
     u32 last, arm, wsum[32];
 };
 template <int KW, int NT, class Sync, bool BINS>
-__device__ __forceinline__ void pass_epilogue(const SelArgs& a, EpilogueSmem& es) {
+__device__ __forceinline__ void pass_epilogue(const SelArgs& a, EpilogueSmem& es, const SelState* planned = nullptr) {
     typedef typename Comp<KW>::t ct;
     Sync::sync();
     if (threadIdx.x == 0) {
@@ -63,9 +71,19 @@ __device__ __forceinline__ void pass_epilogue(const SelArgs& a, EpilogueSmem& es
         __threadfence();
         g->cnt_a = atomic_read(&g->cnt_a);
         g->cnt_b = atomic_read(&g->cnt_b);
+        if (planned) {
+            g->pl = planned->pl;
+            g->pr = planned->pr;
+            g->dst = planned->dst;
+            g->level = planned->level;
+            g->levels_grid = planned->levels_grid;
+            g->pending = 1;
+        }
         decide(*g);
         *a.pass_done = 0;
-        es.arm = a.bins && g->src != SRC_INPUT && g->m_src > a.list_max && g->phase == PH_RUN;
+        g->cnt_a = 0; // for a pass that plans for itself
+        g->cnt_b = 0;
+        es.arm = a.bins && g->m_win > a.list_max && g->phase == PH_RUN && (g->src != SRC_INPUT || g->overflows != 0);
     }
     if constexpr (BINS) {
         Sync::sync();
@@ -88,11 +106,11 @@ __device__ __forceinline__ void pass_epilogue(const SelArgs& a, EpilogueSmem& es
         if (lane == 31) es.wsum[warp] = incl;
         Sync::sync();
         for (u32 w = 0; w < warp; ++w) incl += es.wsum[w];
-        const u32 r = (u32)(*(volatile u64*)&g->k_rem - 1), nb = (u32) * (volatile u64*)&g->m_src;
+        const u32 r = (u32)(*(volatile u64*)&g->k_rem - 1), nb = (u32) * (volatile u64*)&g->m_win;
         u32 run = incl - t;
 #pragma unroll
         for (u32 q = 0; q < PER; ++q) {
-            if (h[q] && r >= run && r < run + h[q] && h[q] < nb) { // one thread at most
+            if (h[q] && r >= run && r < run + h[q] && h[q] < nb && h[q] <= a.cap_b) { // one thread at most
                 const u32 b = threadIdx.x * PER + q;
                 const u32 sh = a.bins->shift;
                 const ct base = Comp<KW>::from128(a.bins->base), lo = Comp<KW>::from128(g->lo), hi = Comp<KW>::from128(g->hi);
@@ -102,9 +120,8 @@ __device__ __forceinline__ void pass_epilogue(const SelArgs& a, EpilogueSmem& es
                 g->pl = (u128)(b == 0 || l < lo ? lo : l);
                 g->pr = (u128)(b == HB_BINS - 1 || u > hi || u < l ? hi : u);
                 g->dst = g->src == SRC_CAND0 ? SRC_CAND1 : SRC_CAND0;
-                g->cnt_a = 0;
-                g->cnt_b = 0;
-                g->dense = run > nb / 16 ? 1u : 0u;
+                // (the input also holds what lies below the window)
+                g->dense = run + (g->src == SRC_INPUT ? g->out_base : 0) > g->m_src / 16 ? 1u : 0u;
                 g->level += 1;
                 g->levels_grid += 1;
                 g->pending = 1;
@@ -179,21 +196,157 @@ template <int DT> __global__ void __launch_bounds__(PASS_NT) k_pass_first(SelArg
     pass_epilogue<KW, PASS_NT, SyncBlock, true>(a, es);
 }
 
-// Second level, over the candidates of the first, when its last block armed it.
-template <int DT> __global__ void __launch_bounds__(PASS_NT) k_pass(SelArgs a) {
+// The pivots of a pass that none has armed, by every block for itself: all draw
+// the same sample and select the same two of its elements, so no block waits for
+// another and no launch is spent on what seldom happens: a bracket that missed
+// rank k, candidates that did not fit their buffer, or bins that resolved nothing.
+// A window that the finish's list (and the buffer) holds is collected as it is.  Otherwise the
+// margin is four standard deviations; where that bracket would not fit the
+// candidate buffer (rank k near an end of a large window) it is drawn from again,
+// up to N * 16 draws of which only those inside it are kept, and its margin
+// narrowed until it is expected to fit.  Sets pl, pr, dst, dense, level of `s`
+// (shared); false: no use (the finish takes the source as it is).
+template <int KW> struct HereSmem {
+    static constexpr u32 N = KW == 32 ? 2048 : 1024;
+    typename Comp<KW>::t samp[N];
+    HistSelSmem<KW> hs;
+    u32 kept, fits;
+    long long jl, jr;
+};
+template <int DT> __device__ __forceinline__ CandSrc<Key<DT>::KW> cand_src(const SelArgs& a, const SelState& s) {
+    const u32 c = s.src == SRC_CAND1 ? 1 : 0;
+    return CandSrc<Key<DT>::KW>{static_cast<const typename Key<DT>::key_t*>(a.cand_key[c]), a.cand_idx[c], s.m_src};
+}
+// Draws from the source of `s`: those inside [lo, hi] are counted, and the first
+// `room` kept in sm.samp.
+template <int DT>
+__device__ __noinline__ u32 here_sample(const SelArgs& a, const SelState& s, typename Comp<Key<DT>::KW>::t lo,
+                                        typename Comp<Key<DT>::KW>::t hi, u32 draws, u32 salt, u32 room,
+                                        HereSmem<Key<DT>::KW>& sm) {
+    if (s.src == SRC_INPUT)
+        block_sample(InputSrc<DT>::make(a.keys, s.m_src), lo, hi, draws, a.parts, a.seed, s.level, salt, sm.samp, room, &sm.kept);
+    else block_sample(cand_src<DT>(a, s), lo, hi, draws, a.parts, a.seed, s.level, salt, sm.samp, room, &sm.kept);
+    const u32 n = sm.kept;
+    __syncthreads();
+    return n;
+}
+template <int DT>
+__device__ __noinline__ bool plan_here(const SelArgs& a, SelState& s, HereSmem<Key<DT>::KW>& sm) {
+    constexpr int KW = Key<DT>::KW;
+    constexpr u32 N = HereSmem<KW>::N, WANT = N / 4 * 3;
+    typedef Comp<KW> C;
+    typedef typename C::t ct;
+    const ct lo = C::from128(s.lo), hi = C::from128(s.hi);
+    ct pl = lo, pr = hi;
+    double below = 0.0; // elements of the window expected below pl
+    if (s.m_win > FIN_LIST<KW> || s.m_win > a.cap_b) {
+        u32 in = 0, under = 0, over = 0; // draws inside [pl, pr], and in the window on either side of it
+        u32 draws = 0;
+        for (u32 stage = 0; stage < 2; ++stage) {
+            // as many draws as leave about WANT inside the bracket
+            const u32 all = in + under + over;
+            const double inside = (stage ? (double)(sm.jr - sm.jl + 2) / (double)all : 1.0) * (double)s.m_win / (double)s.m_src;
+            const double want = (double)WANT / (inside > 0.0 ? inside : 1.0);
+            const u32 most = N * (stage ? 16 : 8), d = want < (double)most ? (u32)want : most;
+            __syncthreads();
+            if (d <= draws) break;
+            draws = d;
+            in = here_sample<DT>(a, s, pl, pr, d, 0x48455245u + stage, N, sm);
+            if (in > N) return false; // (the blocks would keep different draws; 13 standard deviations off)
+            if (in == 0) break; // (nothing learnt)
+            if (stage) {
+                under = pl > lo ? here_sample<DT>(a, s, lo, (ct)(pl - 1), d, 0x48455245u + stage, 0, sm) : 0;
+                over = pr < hi ? here_sample<DT>(a, s, (ct)(pr + 1), hi, d, 0x48455245u + stage, 0, sm) : 0;
+            }
+            if (threadIdx.x == 0) {
+                const u32 n = in + under + over;
+                long long l, r;
+                float z = 4.0f;
+                do {
+                    pivot_ranks(n, s.m_win, s.k_rem, z, false, l, r);
+                    l = l < -1 ? -1 : l;
+                    r = r < n ? r : n;
+                    z *= 0.5f;
+                    sm.fits = (double)(r - l + 1) * (double)s.m_win <= 0.75 * (double)n * (double)a.cap_b;
+                } while (stage && !sm.fits && z > 0.25f);
+                sm.jl = l;
+                sm.jr = r;
+            }
+            __syncthreads();
+            const u32 fits = sm.fits;
+            const long long jl = sm.jl - under, jr = sm.jr - under, top = (long long)in - 1;
+            const u32 r1 = (u32)(jr < 0 ? 0 : jr > top ? top : jr), r0 = jl < 0 ? r1 : (u32)(jl > top ? top : jl);
+            ct x0, x1;
+            block_select_two<KW, PASS_NT>(sm.samp, in, pl, pr, r0, r1, sm.hs, x0, x1);
+            below = sm.jl < 0 ? 0.0 : (double)(sm.jl + 1) * (double)s.m_win / (double)(in + under + over);
+            if (jl >= 0) pl = x0;
+            if (jr <= top) pr = x1;
+            if (fits) break;
+        }
+    }
+    if (pl == lo && pr == hi && s.m_win > a.cap_b) return false;
+    // (the input also holds what lies below the window)
+    if (s.src == SRC_INPUT) below += (double)s.out_base;
+    const u32 dense = below * 16.0 > (double)s.m_src ? 1u : 0u;
+    __syncthreads(); // `s` has been read, and the planning's memory is free again
+    if (threadIdx.x == 0) {
+        s.pl = (u128)pl;
+        s.pr = (u128)pr;
+        s.dense = dense;
+        s.dst = s.src == SRC_CAND0 ? SRC_CAND1 : SRC_CAND0;
+        s.level += 1;
+        s.levels_grid += 1;
+    }
+    __syncthreads();
+    return true;
+}
+
+// The second level where it is not simply the armed pass over the candidates (out
+// of line: its registers would weigh on that one).
+template <int DT>
+__device__ __noinline__ void pass_again(const SelArgs& a, bool armed, HereSmem<Key<DT>::KW>& here,
+                                        WarpQ<Key<DT>::KW>* wq, PassSmem<PASS_NT>& ps, EpilogueSmem& es) {
+    typedef Comp<Key<DT>::KW> C;
+    __shared__ SelState s;
+    if (threadIdx.x == 0) s = *a.st;
+    __syncthreads();
+    if (!armed && !plan_here<DT>(a, s, here)) return;
+    const typename C::t lo = C::from128(s.lo), pl = C::from128(s.pl), pr = C::from128(s.pr);
+    const Sink<DT> sink = make_sink<DT>(a, s);
+    WarpQ<Key<DT>::KW>& q = wq[threadIdx.x >> 5];
+    if (s.src == SRC_INPUT)
+        pass_any<PASS_NT, DT>(InputSrc<DT>::make(a.keys, s.m_src), s.dense != 0, lo, pl, pr, sink, ps, q, NoBins{});
+    else pass_any<PASS_NT, DT>(cand_src<DT>(a, s), s.dense != 0, lo, pl, pr, sink, ps, q, NoBins{});
+    pass_epilogue<Key<DT>::KW, PASS_NT, SyncBlock, false>(a, es, armed ? nullptr : &s);
+}
+
+// Second level: over the candidates of the first, or over the input again, when the
+// first's last block armed it or more is left than the finish holds.
+template <int DT> __global__ void __launch_bounds__(PASS_NT, Key<DT>::KW == 32 ? 3 : 2) k_pass(SelArgs a) {
     typedef Key<DT> K;
     constexpr int KW = K::KW;
     typedef Comp<KW> C;
+    union Smem {
+        WarpQ<KW> wq[PASS_NT / 32];
+        HereSmem<KW> here;
+        __device__ Smem() {}
+    };
     __shared__ PassSmem<PASS_NT> ps;
-    __shared__ WarpQ<KW> wq[PASS_NT / 32];
+    __shared__ __align__(16) unsigned char smem_raw[sizeof(Smem)];
+    static_assert(sizeof(Smem) == sizeof(WarpQ<KW>) * (PASS_NT / 32), "planning takes no more than the pass");
+    Smem& sm = *reinterpret_cast<Smem*>(smem_raw);
     __shared__ EpilogueSmem es;
     grid_dep_wait();
     grid_dep_release();
     const SelState s = *a.st;
-    if (s.phase != PH_RUN || !s.pending || s.src == SRC_INPUT) return;
-    const CandSrc<KW> src{static_cast<const typename K::key_t*>(a.cand_key[s.src - 1]), a.cand_idx[s.src - 1], s.m_src};
-    pass_any<PASS_NT, DT>(src, s.dense != 0, C::from128(s.lo), C::from128(s.pl), C::from128(s.pr), make_sink<DT>(a, s),
-                          ps, wq[threadIdx.x >> 5], NoBins{});
+    if (s.phase != PH_RUN) return;
+    if (!s.pending && s.m_src <= FIN_LIST<KW>) return;
+    if (!s.pending || s.src == SRC_INPUT) {
+        pass_again<DT>(a, s.pending != 0, sm.here, sm.wq, ps, es);
+        return;
+    }
+    pass_any<PASS_NT, DT>(cand_src<DT>(a, s), s.dense != 0, C::from128(s.lo), C::from128(s.pl), C::from128(s.pr),
+                          make_sink<DT>(a, s), ps, sm.wq[threadIdx.x >> 5], NoBins{});
     pass_epilogue<KW, PASS_NT, SyncBlock, false>(a, es);
 }
 

@@ -1,0 +1,90 @@
+"""A first level that leaves too much: a bracket that misses rank k, on either
+side, and candidates that do not fit their buffer.  The
+standing second pass then plans for itself (or reads the input again between the
+ends of rank k's bin), so the statistics show a second grid level; the selected
+set and the rank-k pair have to be exact whatever was missed."""
+import numpy as np
+import pytest
+
+import oracle
+
+from _gpu import bits_of, to_device
+from test_select_gpu import keys_for
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def tk():
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_1502_03942_gb300 as tk
+    return tk
+
+
+@pytest.fixture(scope="module")
+def ctx(tk):
+    c = tk.Context(0)
+    yield c
+    c.close()
+
+
+def check(tk, ctx, orc, keys, name, d, k, **kw):
+    """Both forms of the call; the statistics of each."""
+    ok, oi, kk, ki = tk.topk_select(ctx, d, k, params=tk.make_params(**kw))
+    stats = [ctx.last_stats()]
+    assert orc.check_selection(keys, name, k, bits_of(oi), int(bits_of(ki)[0]), out_keys=bits_of(ok),
+                               kth_key=bits_of(kk)) == 0
+    k2, i2 = tk.topk_select_kth(ctx, d, k, params=tk.make_params(**kw))
+    stats.append(ctx.last_stats())
+    assert int(bits_of(k2)[0]) == int(bits_of(kk)[0]) and int(bits_of(i2)[0]) == int(bits_of(ki)[0])
+    return stats
+
+
+@pytest.mark.parametrize("name", ["u32", "i32", "f32", "bf16", "u64"])
+@pytest.mark.parametrize("n,skip", [(140000, 0), ((1 << 20) + 77, 1), ((1 << 22) + 5, 0)])
+def test_missed_bracket(tk, ctx, name, n, skip):
+    orc = oracle.default()
+    keys = keys_for(name, n + skip, seed=n + 1)
+    d = to_device(keys, name)[skip:]
+    keys = keys[skip:].copy()
+    missed = 0
+    for k in (n // 500, n // 3, 2 * n // 3, n - n // 500):
+        for seed in (1, 2, 3):
+            for s in check(tk, ctx, orc, keys, name, d, k, delta_factor=0.25, flags=tk.TOPK_FLAG_RAW_DELTA, seed=seed):
+                if s["pivot_failures"]:
+                    missed += 1
+                    assert s["levels_grid"] >= 2, (k, seed, s)
+    assert missed > 0
+
+
+@pytest.mark.parametrize("name", ["u32", "f32", "u64"])
+@pytest.mark.parametrize("n,skip", [((1 << 20) + 77, 1), ((1 << 22) + 5, 0), (1 << 24, 0)])
+def test_overflowed_candidates(tk, ctx, name, n, skip):
+    orc = oracle.default()
+    keys = keys_for(name, n + skip, seed=n + 2)
+    d = to_device(keys, name)[skip:]
+    keys = keys[skip:].copy()
+    over = 0
+    for k in (n // 5, n // 2, n - n // 5):
+        for s in check(tk, ctx, orc, keys, name, d, k, flags=tk.TOPK_FLAG_TINY_CAND):
+            if s["overflows"]:
+                over += 1
+                assert s["levels_grid"] >= 2, (k, s)
+    assert over > 0
+
+
+def test_small_margins_on_large_inputs(tk, ctx):
+    """The documented setting: brackets of one standard deviation, which miss
+    about one call in three, at a size whose second plan stands ready and at one
+    whose does not."""
+    orc = oracle.default()
+    for n in ((1 << 23) + 1, 1 << 25):
+        keys = keys_for("f32", n, seed=9)
+        d = to_device(keys, "f32")
+        missed = 0
+        for seed in range(1, 7):
+            for s in check(tk, ctx, orc, keys, "f32", d, n // 3, delta_factor=1.0, seed=seed):
+                missed += s["pivot_failures"] > 0
+                assert s["pivot_failures"] == 0 or s["levels_grid"] >= 2
+        assert missed > 0
