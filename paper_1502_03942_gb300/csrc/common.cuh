@@ -227,6 +227,7 @@ struct SelArgs {
     u32 list_max;             // undecided elements that the finish takes without a second pass
     int first_dense;          // first level's pass mode chosen by the host (0/1), or -1
     u32 kth_only;             // only the rank-k pair is wanted: no selected element is written
+    u32 plan_follows;         // a level by sampling stands behind the second pass
 };
 
 

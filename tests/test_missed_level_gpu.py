@@ -1,5 +1,5 @@
 """A first level that leaves too much: a bracket that misses rank k, on either
-side, and candidates that do not fit their buffer.  The
+side, candidates that do not fit their buffer, and bins that part nothing.  The
 standing second pass then plans for itself (or reads the input again between the
 ends of rank k's bin), so the statistics show a second grid level; the selected
 set and the rank-k pair have to be exact whatever was missed."""
@@ -88,3 +88,18 @@ def test_small_margins_on_large_inputs(tk, ctx):
                 missed += s["pivot_failures"] > 0
                 assert s["pivot_failures"] == 0 or s["levels_grid"] >= 2
         assert missed > 0
+
+
+@pytest.mark.parametrize("n", [1 << 23, (1 << 24) + 3])
+def test_bins_that_part_nothing(tk, ctx, n):
+    """Half of the keys close to 1, the others up to 1e20 and beyond, rank k just
+    inside the cluster: the bracket reaches over the gap and one bin holds nearly
+    all candidates."""
+    orc = oracle.default()
+    g = np.random.Generator(np.random.Philox(n))
+    keys = np.where(g.random(n) < 0.5, 1 + 1e-6 * g.standard_normal(n), np.exp(g.standard_normal(n)) * 1e20)
+    keys = keys.astype(np.float32).view(np.uint32)
+    d = to_device(keys, "f32")
+    for k in (n // 2 - n // 100, n // 2, n // 2 + n // 100):
+        check(tk, ctx, orc, keys, "f32", d, k)
+        check(tk, ctx, orc, keys, "f32", d, k, flags=tk.TOPK_FLAG_TINY_CAND)
