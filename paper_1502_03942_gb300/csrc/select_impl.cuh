@@ -927,7 +927,7 @@ __global__ void __launch_bounds__(EXT_NT) k_extreme(SelArgs a, u32* counter, voi
     raw_t* ok_out = static_cast<raw_t*>(a.out_keys);
     ct best = want_max ? (ct)0 : C::max_value();
     constexpr u64 TILE = (u64)EXT_NT * 16;
-    const u64 ntiles = (a.n + TILE - 1) / TILE;
+    const u64 ntiles = (src.extent() + TILE - 1) / TILE; // (an input that starts inside 16 bytes reaches further)
     for (u64 t = blockIdx.x; t < ntiles; t += gridDim.x) {
         typename K::key_t kk[16];
         u32 ii[16];
