@@ -455,8 +455,9 @@ template <int DT> __global__ void __launch_bounds__(CL_NT) k_plan(SelArgs a, int
 
 // ------------------------------------------------------------- the finish
 
-// The source that one block finishes alone: 8 us up to this size, where a
-// cluster takes 12 for the same elements (its barriers and remote accesses).
+// What is left of a source that one block of the cluster finishes alone: 8 us up
+// to this size, where all of them take 12 for the same elements (their barriers
+// and remote accesses).
 constexpr u32 FIN_SOLO = 4096;
 
 template <int KW> struct FinSmem {

@@ -15,7 +15,8 @@
 //                        sampling for candidates that the bins did not part
 //   k_finish (1 cluster) selection of rank k among what is left, the rest of
 //                        the output and the rank-k pair
-// Inputs of at most T keys take k_finish alone.
+// Inputs of at most T keys take one launch: k_small (1 block) up to SMALL_MAX keys,
+// k_finish above.
 // Each recursion level used to sample anew (k_sample, k_pivots: about 17 us) before
 // its pass, two or three times a call; the bins give the second level exact
 // counts for nothing and narrow by a factor of about 1000 instead of 30.
@@ -875,6 +876,22 @@ __global__ void __launch_bounds__(TMA_NT, (TmaCfg<DT, MODE>::MIN_BLOCKS)) k_pass
     pass_epilogue<KW, TMA_CONS, SyncNamed<1, TMA_CONS>, true>(a, es);
 }
 
+// A short input whole, in one block: its keys into shared memory, rank k by a
+// histogram over the key domain, the elements up to it written.  The cluster of
+// k_finish is slower on so few (its barriers and its range step): 100 keys 5.4 us
+// here, 6.3 by its first block alone; 8192 normal f32 keys 10.5 here, 12.6 by all
+// eight, which pay from about 12000 keys on.
+constexpr u32 SMALL_MAX = 8192;
+template <int DT> using SmallSmem = BlockSmem<Key<DT>::KW, BLK_NT, SMALL_MAX>;
+template <int DT> __global__ void __launch_bounds__(BLK_NT) k_small(SelArgs a) {
+    grid_dep_wait();
+    grid_dep_release();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    if (threadIdx.x == 0) init_state<DT>(a.st, a);
+    __syncthreads();
+    block_finish<DT>(a, *reinterpret_cast<SmallSmem<DT>*>(smem_raw));
+}
+
 // k = 1: the minimum pair (base case of Algorithm "select");
 // k = n: every pair, plus the maximum as the rank-n pair.
 template <int KW> __device__ __forceinline__ typename Comp<KW>::t shfl_xor_ct(typename Comp<KW>::t v, int o);
@@ -1051,7 +1068,9 @@ template <int DT> static topk_status set_smem_attrs() {
     if (cudaFuncSetAttribute(k_plan<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)sizeof(PlanSmem<Key<DT>::KW>)) != cudaSuccess ||
         cudaFuncSetAttribute(k_finish<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)sizeof(FinSmem<Key<DT>::KW>)) != cudaSuccess)
+                             (int)sizeof(FinSmem<Key<DT>::KW>)) != cudaSuccess ||
+        cudaFuncSetAttribute(k_small<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SmallSmem<DT>)) !=
+            cudaSuccess)
         return TOPK_ECUDA;
     done_mask.fetch_or(bit);
     return TOPK_OK;
@@ -1172,8 +1191,8 @@ static topk_status enqueue_select(topk_ctx* ctx, SelArgs a, const Tuning& tu, in
         }
         if (e != cudaSuccess) return cuda_status(e);
     }
-    const int fin = one && n <= FIN_SOLO ? 1 : CL_BLOCKS; // (the kernel leaves a short source to one block)
-    e = launch_dep(k_finish<DT>, fin, CL_NT, sizeof(FinSmem<KW>), st, fin, a, one ? 1 : 0);
+    if (one && n <= SMALL_MAX) e = launch_dep(k_small<DT>, 1, BLK_NT, sizeof(SmallSmem<DT>), st, 1, a);
+    else e = launch_dep(k_finish<DT>, CL_BLOCKS, CL_NT, sizeof(FinSmem<KW>), st, CL_BLOCKS, a, one ? 1 : 0);
     if (e != cudaSuccess) return cuda_status(e);
     if (ctx) count_launch(ctx, one ? 1 : resample ? 6 : 4);
     return cuda_status(cudaGetLastError());
