@@ -360,10 +360,12 @@ template <int DT> struct Sink {
 // composite, so that the bins of a bracket of few distinct keys are not spent on
 // positions that no element has.
 struct NoBins {
+    static constexpr bool COUNTS = false;
     template <class K> __device__ __forceinline__ void add(K, u32) const {}
 };
 template <int KW> struct BinHist {
     typedef typename Comp<KW>::t ct;
+    static constexpr bool COUNTS = true;
     u32* h;
     ct base;
     u32 sh, bn;
@@ -636,6 +638,19 @@ __device__ __forceinline__ void tile_count_dispatch(const typename Key<DT>::raw_
     }
 }
 
+// r[q] for a lane-dependent q without dynamic register indexing (which would
+// move r to local memory): a tree of selects.
+template <class T> __device__ __forceinline__ T pick16(const T (&r)[16], u32 q) {
+    T l1[8], l2[4], l3[2];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) l1[j] = (q & 1u) ? r[2 * j + 1] : r[2 * j];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) l2[j] = (q & 2u) ? l1[2 * j + 1] : l1[2 * j];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) l3[j] = (q & 4u) ? l2[2 * j + 1] : l2[2 * j];
+    return (q & 8u) ? l3[1] : l3[0];
+}
+
 // ------------------------------------------------------------ the pass
 // Streams the source in tiles of NT*16 elements, classifies every element
 // against (lo, pl, pr) and compacts a and b.  A tile with neither costs one
@@ -770,6 +785,30 @@ __device__ __forceinline__ void classify_emit(const KeyT (&kk)[16], PosF pos, u3
             }
         }
     }
+    if constexpr (Bins::COUNTS) {
+        // few elements, each counted as well: a lane writes its own (unrolled over the
+        // slots like the others, the counting took 14 registers more, and with them
+        // one of four resident blocks)
+        if (__any_sync(0xffffffffu, mb)) {
+            const u32 cnt = (u32)__popc(mb);
+            u32 incl = cnt;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const u32 y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= (u32)o) incl += y;
+            }
+            rb += incl - cnt;
+            while (mb) {
+                const u32 q = (u32)(__ffs(mb) - 1);
+                mb &= mb - 1;
+                const KeyT key = pick16(kk, q);
+                const u32 x = pos((int)q);
+                sink.put_b(rb++, key, x);
+                bins.add(key, x);
+            }
+        }
+        return;
+    }
     if (__any_sync(0xffffffffu, mb)) {
         if (rb + wb <= sink.cap_b) {
             auto* bkp = sink.ck + rb;
@@ -783,7 +822,6 @@ __device__ __forceinline__ void classify_emit(const KeyT (&kk)[16], PosF pos, u3
                 if (bit) {
                     bkp[r] = kk[s];
                     bip[r] = x;
-                    bins.add(kk[s], x);
                 }
                 const u32 c = (u32)__popc(bal);
                 bkp += c;
@@ -793,10 +831,7 @@ __device__ __forceinline__ void classify_emit(const KeyT (&kk)[16], PosF pos, u3
 #pragma unroll
             for (int s = 0; s < 16; ++s) {
                 const u32 bal = __ballot_sync(0xffffffffu, (mb >> s) & 1u);
-                if ((mb >> s) & 1u) {
-                    sink.put_b(rb + __popc(bal & below), kk[s], pos(s));
-                    bins.add(kk[s], pos(s));
-                }
+                if ((mb >> s) & 1u) sink.put_b(rb + __popc(bal & below), kk[s], pos(s));
                 rb += __popc(bal);
             }
         }
@@ -957,19 +992,6 @@ __device__ __forceinline__ void lq_append(u32 hit, PosF pos, KeyAt key_at, typen
         ++qs.cnt;
     }
 }
-// r[q] for a lane-dependent q without dynamic register indexing (which would
-// move r to local memory): a tree of selects.
-template <class T> __device__ __forceinline__ T pick16(const T (&r)[16], u32 q) {
-    T l1[8], l2[4], l3[2];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) l1[j] = (q & 1u) ? r[2 * j + 1] : r[2 * j];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) l2[j] = (q & 2u) ? l1[2 * j + 1] : l1[2 * j];
-#pragma unroll
-    for (int j = 0; j < 2; ++j) l3[j] = (q & 4u) ? l2[2 * j + 1] : l2[2 * j];
-    return (q & 8u) ? l3[1] : l3[0];
-}
-
 // Register path in sparse mode.
 template <int NT, int DT, class Src, class Bins>
 __device__ void pass_tiles_sparse(const Src& src, u64 tile0, u64 tile_step, typename Comp<Src::KW>::t lo,

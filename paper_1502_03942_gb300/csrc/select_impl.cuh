@@ -181,25 +181,35 @@ __device__ __forceinline__ void pass_any(const Src& src, bool dense, typename Co
     else pass_tiles<NT, true, false, DT>(src, blockIdx.x, gridDim.x, lo, pl, pr, sink, ps, bins);
 }
 
-// First level on misaligned input.
-template <int DT> __global__ void __launch_bounds__(PASS_NT) k_pass_first(SelArgs a) {
+// First level on misaligned input.  Streams best with four blocks on an SM: the bins'
+// place and width stay in shared memory, read where an element is counted, which
+// leaves the 64 registers that takes.  2^28 f32 keys at k = n / 3: 808 us a call, 1039
+// with three blocks and the bins in registers.
+template <int KW> struct SmemBins {
+    static constexpr bool COUNTS = true;
+    u32 h[HB_BINS];
+    BinHist<KW> b;
+    __device__ __forceinline__ void add(typename Comp<KW>::key_t k, u32 x) const { b.add(k, x); }
+};
+template <int DT> __global__ void __launch_bounds__(PASS_NT, Key<DT>::KW == 32 ? 4 : 2) k_pass_first(SelArgs a) {
     constexpr int KW = Key<DT>::KW;
     typedef Comp<KW> C;
     __shared__ PassSmem<PASS_NT> ps;
     __shared__ WarpQ<KW> wq[PASS_NT / 32];
-    __shared__ u32 hist[HB_BINS];
+    __shared__ __align__(16) unsigned char bins_raw[sizeof(SmemBins<KW>)];
+    auto& bins = *reinterpret_cast<SmemBins<KW>*>(bins_raw);
     __shared__ EpilogueSmem es;
-    for (u32 i = threadIdx.x; i < HB_BINS; i += PASS_NT) hist[i] = 0;
+    for (u32 i = threadIdx.x; i < HB_BINS; i += PASS_NT) bins.h[i] = 0;
     grid_dep_wait();
     const SelState s = *a.st;
     if (s.phase != PH_RUN || !s.pending || s.src != SRC_INPUT) return;
+    if (threadIdx.x == 0) bins.b = make_bins<DT>(a, bins.h);
     __syncthreads();
-    const BinHist<KW> bins = make_bins<DT>(a, hist);
     pass_any<PASS_NT, DT>(InputSrc<DT>::make(a.keys, s.m_src), s.dense != 0, C::from128(s.lo), C::from128(s.pl),
                           C::from128(s.pr), make_sink<DT>(a, s), ps, wq[threadIdx.x >> 5], bins);
     grid_dep_release();
     __syncthreads();
-    add_bins<PASS_NT>(a, hist);
+    add_bins<PASS_NT>(a, bins.h);
     pass_epilogue<KW, PASS_NT, SyncBlock, true>(a, es);
 }
 
