@@ -295,11 +295,13 @@ template <int KW> __device__ __forceinline__ u32* pool_idx(const BatchArgs& b, u
 // same pass took 912 us (68 us of each are the program's own).
 constexpr int ROWS_NT = 256;
 constexpr u32 ROWS_DRAW = 128;  // keys per draw of the sample
-constexpr int ROWS_PER_SM = 3; // resident blocks (registers and shared memory)
 constexpr u64 ROWS_MAX = 1ull << 19; // longest row: beyond, one block's read takes longer than the general path
 template <int KW> struct RowsCfg {
     static constexpr u32 CAP = KW == 32 ? 4096 : 2048; // elements of the list (32 KB)
     static constexpr u32 KMAX = CAP / 2;               // largest k: cutting back frees half the list
+    // resident blocks: 64-bit keys spill 300 bytes of the 80 registers that three
+    // leave (4096 rows of 2^U(10, 18) u64 keys 542 us with three, 395 with two)
+    static constexpr int PER_SM = KW == 32 ? 3 : 2;
 };
 
 template <int KW> struct RowsSmem {
@@ -362,7 +364,7 @@ template <int KW> __device__ __noinline__ void rows_cut(RowsSmem<KW>& sm, u32 ha
     __syncthreads();
 }
 
-template <int DT> __global__ void __launch_bounds__(ROWS_NT, ROWS_PER_SM) k_rows(BatchArgs b) {
+template <int DT> __global__ void __launch_bounds__(ROWS_NT, RowsCfg<Key<DT>::KW>::PER_SM) k_rows(BatchArgs b) {
     grid_dep_wait();
     typedef Key<DT> K;
     typedef typename K::raw_t raw_t;
@@ -1043,7 +1045,7 @@ static topk_status launch_batched(topk_ctx* ctx, BatchArgs b, cudaStream_t st) {
     int pass_per_sm = 1, plan_per_sm = 1;
     if (b.split != WIDE_NONE && (rs = wide_setup<DT>(ctx->device, pass_per_sm, plan_per_sm)) != TOPK_OK) return rs;
     // rows that all start at once need no order
-    b.ordered = b.rows > (u32)ctx->sms * ROWS_PER_SM;
+    b.ordered = b.rows > (u32)ctx->sms * RowsCfg<KW>::PER_SM;
     const bool order = b.ordered || !b.rest;
     cudaError_t e = order ? launch_dep(k_batch_order, 1, 1024, 0, st, 1, b) : cudaSuccess;
     if (e == cudaSuccess && b.rest) {
@@ -1055,7 +1057,7 @@ static topk_status launch_batched(topk_ctx* ctx, BatchArgs b, cudaStream_t st) {
                 return TOPK_ECUDA;
             attr.fetch_or(bit);
         }
-        const int grid = (int)std::min<u64>(b.rows, (u64)ctx->sms * ROWS_PER_SM);
+        const int grid = (int)std::min<u64>(b.rows, (u64)ctx->sms * RowsCfg<KW>::PER_SM);
         e = launch_dep(k_rows<DT>, grid, ROWS_NT, sizeof(RowsSmem<KW>), st, 1, b);
     }
     if (e == cudaSuccess && b.split != WIDE_NONE) {
