@@ -76,11 +76,13 @@ struct BatchArgs {
     void* const* row_kth_key;
     u32* const* row_kth_idx;
     u32* order;         // rows: row ids, longest first
+    u32* mine;          // rows: those that k_rows takes, when it does not take them all
     u32* rest;          // rows left to the general path by k_rows (null: all rows)
     u32* nrest;         // their number (zero between calls)
-    u32* rows_done;     // blocks of k_rows or k_batched that are done (zero between kernels)
+    u32 sms;
+    u32* rows_done;     // blocks of k_rows that are done (zero between kernels)
     u32 ordered;        // k_rows takes the rows in `order` from the queue, else row i in block i
-    u32* queue;         // next index into order (zero between kernels)
+    u32* queue;         // next index into order (zero from order_rows on)
     SelState* states;   // one per block
     char* cand;         // per block: key'[2][CAP], idx[2][CAP]
     u64 seed;
@@ -92,7 +94,7 @@ struct BatchArgs {
     u32 key_bytes;      // width of a key
     u32 split;          // rows longer than this are wide
     u32* wide;          // rows: ids of the wide rows, longest first
-    u32* words;         // [0] wide rows, [1] planning queue, [2] rows in order
+    u32* words;         // [0] wide rows, [1] planning queue, [2] rows in order, [3] rows that k_rows takes
     u64* tile_pre;      // rows + 1: tiles of the wide rows before the j-th
     u32* done;          // rows: tiles of the row classified by the wide pass
     SelState* rstate;   // rows: state of each wide row
@@ -175,6 +177,7 @@ __device__ void order_rows(const BatchArgs& b, const u32* src, u32 rows, bool li
             run += hist[k];
         }
         b.words[2] = rows;
+        *b.queue = 0;
     }
     __syncthreads();
     for (u32 i0 = threadIdx.x; i0 < rows; i0 += U * blockDim.x) {
@@ -238,10 +241,117 @@ __device__ void order_rows(const BatchArgs& b, const u32* src, u32 rows, bool li
     }
 }
 
-__global__ void __launch_bounds__(1024) k_batch_order(BatchArgs b) {
+constexpr int ROWS_NT = 256;
+constexpr u32 ROWS_DRAW = 128;  // keys per draw of the sample
+constexpr u64 ROWS_MAX = 1ull << 19; // longest row: beyond, one block's read takes longer than the general path
+template <int KW> struct RowsCfg {
+    static constexpr u32 CAP = KW == 32 ? 4096 : 2048; // elements of the list (32 KB)
+    static constexpr u32 KMAX = CAP / 2;               // largest k: cutting back frees half the list
+    // resident blocks: 64-bit keys spill 300 bytes of the 80 registers that three
+    // leave (4096 rows of 2^U(10, 18) u64 keys 542 us with three, 395 with two)
+    static constexpr int PER_SM = KW == 32 ? 3 : 2;
+};
+
+// Which rows k_rows (below) takes: one block reads such a row whole, at about 8.5
+// keys per ns, while the general path spreads a long row over the whole GPU for
+// about 42 us (its launches and barriers) and, in all, some 1e6 keys a us.  So a long
+// row pays only in a batch that keeps the GPU busy with the others: the longest may
+// exceed 7/8 of 2^17 keys by 1/128 of the batch's, and by 2^18 where the general
+// path would also have to run blocks of its own for rows just below the split
+// length, or for more rows than two waves of them.  When a row is longer than that,
+// or its k too large, the general path runs in any case; then rows up to 1/256 of
+// the keys that k_rows could take are still worth it (they save the general path
+// more than they take), and rows up to the split length where that takes all its
+// one-block work away or they are many.
+// us by k_rows / by the general path, f32, k = 100: 1 row of 2^17 43 / 41, of 2^19
+// 82 / 43; 64 rows of 2^18 59 / 66, of 2^19 101 / 88; 128 rows of 2^19 106 / 112; 64 rows
+// of 2^U(10, 18) 53 / 73; 4000 rows of 2000 keys and 4 of 2^18 107 / 387.
+struct RowsPlan {
+    u32 longest, shortest, nshort, flags;
+    u64 keys;
+};
+// The longest row that k_rows takes (0: it takes none).  All NT threads call.
+template <int KW, int NT> __device__ u32 rows_limit(const BatchArgs& b, RowsPlan& p) {
+    enum : u32 { LEFT = 1, MID = 2, MID_LEFT = 4 }; // rows left whatever the limit; rows of 2^13 keys to the split length
+    if (b.row_keys || b.split == WIDE_NONE) return (u32)ROWS_MAX; // (no row is spread over the GPU)
+    if (threadIdx.x == 0) p = RowsPlan{0u, 0xFFFFFFFFu, 0u, 0u, 0ull};
+    __syncthreads();
+    u32 mx = 0, mn = 0xFFFFFFFFu, ns = 0, fl = 0;
+    u64 sum = 0;
+    for (u32 i = threadIdx.x; i < b.rows; i += NT) {
+        const u64 n = row_len(b, i), k = b.row_k[i];
+        if (k == 0 || k > n || n > 0xFFFFFFFFull) {
+            mn = 0; // (reported by whoever takes it)
+            continue;
+        }
+        const bool mid = n > 8192 && n <= b.split;
+        if (n > RowsCfg<KW>::CAP && k > RowsCfg<KW>::KMAX) {
+            fl |= mid ? LEFT | MID_LEFT : LEFT;
+            continue;
+        }
+        fl |= (mid ? MID : 0u) | (n > ROWS_MAX ? LEFT : 0u);
+        ns += (u32)(n <= b.split);
+        sum += n <= ROWS_MAX ? n : 0;
+        mx = max(mx, (u32)n);
+        mn = min(mn, (u32)n);
+    }
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    mn = __reduce_min_sync(0xffffffffu, mn);
+    ns = __reduce_add_sync(0xffffffffu, ns);
+    fl = __reduce_or_sync(0xffffffffu, fl);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, (unsigned long long)sum, o);
+    if (lane_id() == 0) {
+        atomicMax(&p.longest, mx);
+        atomicMin(&p.shortest, mn);
+        atomicAdd(&p.nshort, ns);
+        atomicOr(&p.flags, fl);
+        atomicAdd(reinterpret_cast<unsigned long long*>(&p.keys), (unsigned long long)sum);
+    }
+    __syncthreads();
+    const u64 total = b.row_off[b.rows] - b.row_off[0];
+    const bool many = p.nshort > 2 * b.sms;
+    u64 limit = ROWS_MAX;
+    if ((p.flags & LEFT) || p.longest > (7ull << 14) + total / 128 + ((p.flags & MID) || many ? 1ull << 18 : 0ull)) {
+        limit = p.keys / 256 < ROWS_MAX ? p.keys / 256 : ROWS_MAX;
+        if (limit < b.split) limit = many || (p.flags & (MID | MID_LEFT)) == MID ? b.split : 0u;
+    }
+    return p.shortest <= limit ? (u32)limit : 0u;
+}
+template <int KW> __device__ __forceinline__ bool rows_takes(u64 n, u64 k, u32 limit) {
+    return n <= limit && (n <= RowsCfg<KW>::CAP || k <= RowsCfg<KW>::KMAX);
+}
+
+// Rows in order for the general path, or, with k_rows (b.rest), the rows that it
+// takes; the others go to its list of those it leaves.
+template <int KW> __global__ void __launch_bounds__(1024) k_batch_order(BatchArgs b) {
     grid_dep_wait();
     grid_dep_release();
-    order_rows<1024>(b, nullptr, b.rows, b.rest == nullptr);
+    if (!b.rest) {
+        order_rows<1024>(b, nullptr, b.rows, true);
+        return;
+    }
+    __shared__ RowsPlan plan;
+    __shared__ u32 nmine, nrest;
+    const u32 limit = rows_limit<KW, 1024>(b, plan);
+    if (limit == 0) {
+        if (threadIdx.x == 0) b.words[3] = 0;
+        order_rows<1024>(b, nullptr, b.rows, true);
+        return;
+    }
+    if (threadIdx.x == 0) nmine = nrest = 0;
+    __syncthreads();
+    for (u32 i = threadIdx.x; i < b.rows; i += 1024) {
+        const u64 n = row_len(b, i), k = b.row_k[i];
+        if (k == 0 || k > n || n > 0xFFFFFFFFull || rows_takes<KW>(n, k, limit)) b.mine[atomicAdd(&nmine, 1u)] = i;
+        else b.rest[atomicAdd(&nrest, 1u)] = i;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        b.words[3] = nmine;
+        *b.nrest = nrest;
+    }
+    order_rows<1024>(b, b.mine, nmine, false);
 }
 
 // Arguments of row `row` (keys at r0, n keys, rank k) for the selection
@@ -277,7 +387,8 @@ template <int KW> __device__ __forceinline__ u32* pool_idx(const BatchArgs& b, u
 }
 
 // ---------------------------------------------------- rows in one read
-// Rows of small k (k_rows), one block per row, rows longest first from a queue.
+// Rows of small k (k_rows; which, see rows_limit), one block per row, rows longest
+// first from a queue.
 // A row of at most CAP keys is gathered whole; a longer one is sampled (about
 // one key in 128), the sample element of rank k|S|/n + Delta is the bound, and
 // the row is streamed once, every element up to the bound going to a list in
@@ -293,23 +404,13 @@ template <int KW> __device__ __forceinline__ u32* pool_idx(const BatchArgs& b, u
 // registers, spilled) 344, two 360, two of 512 threads 376.  By levels, whose wide
 // rows went through memory three times and whose blocks waited on barriers, the
 // same pass took 912 us (68 us of each are the program's own).
-constexpr int ROWS_NT = 256;
-constexpr u32 ROWS_DRAW = 128;  // keys per draw of the sample
-constexpr u64 ROWS_MAX = 1ull << 19; // longest row: beyond, one block's read takes longer than the general path
-template <int KW> struct RowsCfg {
-    static constexpr u32 CAP = KW == 32 ? 4096 : 2048; // elements of the list (32 KB)
-    static constexpr u32 KMAX = CAP / 2;               // largest k: cutting back frees half the list
-    // resident blocks: 64-bit keys spill 300 bytes of the 80 registers that three
-    // leave (4096 rows of 2^U(10, 18) u64 keys 542 us with three, 395 with two)
-    static constexpr int PER_SM = KW == 32 ? 3 : 2;
-};
-
 template <int KW> struct RowsSmem {
     typename Comp<KW>::t list[RowsCfg<KW>::CAP];
     HistSelSmem<KW> hs;
     u32 n, full_at, full, row, out;
     u32 last; // the block is the kernel's last (a word of its own: `row` may still be read)
     u32 lead[2][ROWS_NT / 32];
+    RowsPlan plan;
     long long rank;
 };
 
@@ -372,7 +473,7 @@ template <int DT> __global__ void __launch_bounds__(ROWS_NT, RowsCfg<Key<DT>::KW
     constexpr int KW = K::KW;
     typedef Comp<KW> C;
     typedef typename C::t ct;
-    constexpr u32 CAP = RowsCfg<KW>::CAP, KMAX = RowsCfg<KW>::KMAX;
+    constexpr u32 CAP = RowsCfg<KW>::CAP;
     constexpr int EPV = InputSrc<DT>::EPV, NV = InputSrc<DT>::NV;
     constexpr u32 SUB = 512; // keys of a warp's step: 16 per lane
     constexpr u32 WARPS = ROWS_NT / 32;
@@ -380,11 +481,22 @@ template <int DT> __global__ void __launch_bounds__(ROWS_NT, RowsCfg<Key<DT>::KW
     auto& sm = *reinterpret_cast<RowsSmem<KW>*>(smem_raw);
     const u32 tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
     const bool by_ptr = b.row_keys != nullptr;
+    const u32 queued = b.ordered ? b.words[3] : 0u;
     auto next_row = [&]() -> u32 {
         if (!b.ordered) return 0xFFFFFFFFu;
         const u32 idx = atomicAdd(b.queue, 1u);
-        return idx < b.rows ? b.order[idx] : 0xFFFFFFFFu;
+        return idx < queued ? b.order[idx] : 0xFFFFFFFFu;
     };
+    u32 limit = (u32)ROWS_MAX; // (rows in order were chosen)
+    if (b.ordered) {
+        if (queued == 0) return;
+    } else {
+        limit = rows_limit<KW, ROWS_NT>(b, sm.plan);
+        if (limit == 0) { // none: one block orders them all for the general path
+            if (blockIdx.x == 0) order_rows<ROWS_NT>(b, nullptr, b.rows, true);
+            return;
+        }
+    }
     u32 ahead = !b.ordered ? blockIdx.x : tid == 0 ? next_row() : 0u; // (no more blocks than rows)
     while (true) {
         if (tid == 0) {
@@ -407,7 +519,7 @@ template <int DT> __global__ void __launch_bounds__(ROWS_NT, RowsCfg<Key<DT>::KW
             continue;
         }
         const bool whole = n64 <= CAP;
-        if (!whole && (n64 > ROWS_MAX || k64 > KMAX)) {
+        if (!rows_takes<KW>(n64, k64, limit)) {
             if (tid == 0) b.rest[atomicAdd(b.nrest, 1u)] = row;
             __syncthreads();
             continue;
@@ -574,7 +686,6 @@ template <int DT> __global__ void __launch_bounds__(ROWS_NT, RowsCfg<Key<DT>::KW
     if (tid == 0) {
         *b.rows_done = 0;
         *b.nrest = 0;
-        *b.queue = 0;
     }
 }
 
@@ -906,24 +1017,19 @@ __global__ void __launch_bounds__(NT, (BatchVariant<Key<DT>::KW, NT>::MINB)) k_b
     constexpr int KW = K::KW;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     auto& sm = *reinterpret_cast<BatchSmem<KW, NT>*>(smem_raw);
-    __shared__ u32 s_row;
+    __shared__ u32 s_row, s_rows;
     SelState* g = b.states + blockIdx.x;
     char* cand = b.cand + (size_t)blockIdx.x * 2 * BATCH_CAP * (sizeof(key_t) + 4);
+    if (threadIdx.x == 0) s_rows = b.words[2];
     while (true) {
         if (threadIdx.x == 0) {
             const u32 idx = atomicAdd(b.queue, 1u);
-            s_row = idx < b.words[2] ? b.order[idx] : 0xFFFFFFFFu;
+            s_row = idx < s_rows ? b.order[idx] : 0xFFFFFFFFu;
         }
         __syncthreads();
         const u32 row = s_row;
         __syncthreads();
-        if (row == 0xFFFFFFFFu) { // the last block leaves the queue as it found it
-            if (threadIdx.x == 0 && atomicAdd(b.rows_done, 1u) == gridDim.x - 1) {
-                *b.rows_done = 0;
-                *b.queue = 0;
-            }
-            break;
-        }
+        if (row == 0xFFFFFFFFu) break;
         const bool by_ptr = b.row_keys != nullptr;
         const u64 r0 = by_ptr ? 0 : b.row_off[row];
         const u64 n = by_ptr ? b.row_n[row] : b.row_off[row + 1] - r0;
@@ -975,7 +1081,7 @@ __global__ void __launch_bounds__(NT, (BatchVariant<Key<DT>::KW, NT>::MINB)) k_b
         a.parts = b.parts;
         a.sample = b.sample;
         a.finish_T = b.finish_T;
-            a.z = b.z;
+        a.z = b.z;
         a.flags = b.flags;
         a.aligned = 0;
         a.err = b.err;
@@ -1047,7 +1153,7 @@ static topk_status launch_batched(topk_ctx* ctx, BatchArgs b, cudaStream_t st) {
     // rows that all start at once need no order
     b.ordered = b.rows > (u32)ctx->sms * RowsCfg<KW>::PER_SM;
     const bool order = b.ordered || !b.rest;
-    cudaError_t e = order ? launch_dep(k_batch_order, 1, 1024, 0, st, 1, b) : cudaSuccess;
+    cudaError_t e = order ? launch_dep(k_batch_order<KW>, 1, 1024, 0, st, 1, b) : cudaSuccess;
     if (e == cudaSuccess && b.rest) {
         static std::atomic<uint64_t> attr{0};
         const uint64_t bit = 1ull << (ctx->device & 63);
@@ -1085,13 +1191,14 @@ template <int DT> static int batched_max_grid(topk_ctx* ctx, topk_status& rs) {
 // Scratch regions of one batched launch over `rows` rows with `grid` blocks
 // (and, with wide rows, the per-row arrays and the candidate pool).
 struct BatchCarve {
-    size_t order, rest, words, states, cand;
+    size_t order, mine, rest, words, states, cand;
     size_t wide, tile_pre, done, rstate, rcand, pool_next, pool;
 };
 template <int DT> static Carve batch_carve(u32 rows, int grid, bool wide, BatchCarve& bc) {
     typedef typename Key<DT>::key_t key_t;
     Carve cv;
     bc.order = cv.take(4ull * rows);
+    bc.mine = cv.take(4ull * rows);
     bc.rest = cv.take(4ull * rows);
     bc.words = cv.take(256);
     bc.states = cv.take(sizeof(SelState) * (size_t)grid);
@@ -1133,6 +1240,8 @@ static topk_status run_batched(topk_ctx* ctx, BatchArgs b, int threads, bool by_
     b.queue = ctx->d_counter + 4;
     b.nrest = ctx->d_counter + 5;
     b.rows_done = ctx->d_counter + 6;
+    b.sms = (u32)ctx->sms;
+    b.mine = reinterpret_cast<u32*>(base + bc.mine);
     b.rest = by_rows ? reinterpret_cast<u32*>(base + bc.rest) : nullptr;
     b.states = reinterpret_cast<SelState*>(base + bc.states);
     b.cand = base + bc.cand;
