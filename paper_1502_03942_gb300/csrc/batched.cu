@@ -1051,7 +1051,7 @@ __global__ void __launch_bounds__(NT, (BatchVariant<Key<DT>::KW, NT>::MINB)) k_b
             a.cand_idx[1] = reinterpret_cast<u32*>(cand + 2 * BATCH_CAP * sizeof(key_t) + BATCH_CAP * 4);
             a.st = gw;
             a.cap_b = gw->cap_b;
-            block_levels_and_finish<DT, false>(a, sm);
+            block_levels_and_finish<DT>(a, sm);
             __syncthreads();
             continue;
         }
@@ -1090,7 +1090,7 @@ __global__ void __launch_bounds__(NT, (BatchVariant<Key<DT>::KW, NT>::MINB)) k_b
             g->phase = PH_FINISH;
         }
         __syncthreads();
-        block_levels_and_finish<DT, false>(a, sm);
+        block_levels_and_finish<DT>(a, sm);
         __syncthreads();
     }
 }

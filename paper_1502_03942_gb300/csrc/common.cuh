@@ -216,7 +216,7 @@ struct SelArgs {
     u64 seed;
     u32 parts;                // sampling partitions
     u32 sample;               // draws per level
-    u32 finish_T;             // single-block finish threshold
+    u32 finish_T;             // single-block finish threshold (block_levels_and_finish)
     float z;                  // pivot margin factor
     u32 flags;
     u32 aligned;              // input is 16-byte aligned

@@ -1,7 +1,8 @@
 // select_block.cuh — one thread block runs whole recursion levels of the
 // selection: planning (sample + pivots), a block-wide pass, the branch, and
 // the final exact selection among at most T candidates.  Used by the batched
-// kernels (batched.cu), where every block selects whole rows.
+// kernels (batched.cu), where every block selects whole rows; the finish also by
+// k_small (select_impl.cuh).
 #pragma once
 
 #include "select_core.cuh"
@@ -50,54 +51,45 @@ __device__ __forceinline__ u32 warp_reserve(u32 cnt, u32* counter) {
     return __shfl_sync(0xffffffffu, base, 31) + incl - cnt;
 }
 
-// All 32 lanes call; returns the slot of this lane's element when `keep`.
-__device__ __forceinline__ u32 warp_append(bool keep, u32* counter) {
-    const u32 bal = __ballot_sync(0xffffffffu, keep);
-    u32 base = 0;
-    if (lane_id() == 0 && bal) base = atomicAdd(counter, (u32)__popc(bal));
-    base = __shfl_sync(0xffffffffu, base, 0);
-    return base + __popc(bal & lanemask_lt());
-}
-
 // The state of a call before its first level.
-template <int DT> __device__ SelState initial_state(const SelArgs& a) {
+template <int DT> __device__ __forceinline__ void init_state(SelState* g, const SelArgs& a) {
+    g->lo = 0;
+    g->hi = key_domain_max<DT>();
+    g->pl = 0;
+    g->pr = 0;
+    g->m_src = a.n;
+    g->m_win = a.n;
+    g->k_rem = a.k;
+    g->out_base = 0;
+    g->cnt_a = 0;
+    g->cnt_b = 0;
+    g->cap_b = a.cap_b;
+    g->first_cand = 0;
+    g->level = 0;
+    g->phase = PH_RUN;
+    g->src = SRC_INPUT;
+    g->dst = SRC_CAND0;
+    g->pending = 0;
+    g->status = ST_OK;
+    g->levels_grid = 0;
+    g->levels_block = 0;
+    g->failures = 0;
+    g->overflows = 0;
+    g->sample_kept = 0;
+    g->dense = 0;
+}
+template <int DT> __device__ __forceinline__ SelState initial_state(const SelArgs& a) {
     SelState s;
-    s.lo = 0;
-    s.hi = key_domain_max<DT>();
-    s.pl = 0;
-    s.pr = 0;
-    s.m_src = a.n;
-    s.m_win = a.n;
-    s.k_rem = a.k;
-    s.out_base = 0;
-    s.cnt_a = 0;
-    s.cnt_b = 0;
-    s.cap_b = a.cap_b;
-    s.first_cand = 0;
-    s.level = 0;
-    s.phase = PH_RUN;
-    s.src = SRC_INPUT;
-    s.dst = SRC_CAND0;
-    s.pending = 0;
-    s.status = ST_OK;
-    s.levels_grid = 0;
-    s.levels_block = 0;
-    s.failures = 0;
-    s.overflows = 0;
-    s.sample_kept = 0;
-    s.dense = 0;
+    init_state<DT>(&s, a);
     return s;
 }
-template <int DT> __device__ void init_state(SelState* g, const SelArgs& a) { *g = initial_state<DT>(a); }
 
 // ------------------------------------------------------------ one pass
 
 // One pass over the source of state `s` (tiles tile0, tile0 + step, ...):
-// a to the output, b to candidate buffer s.dst, the counts reserved on
-// *cnt_a and *cnt_b.
-template <int NT, int DT, bool INPUT_ONLY = false, bool ONLY_EXACT = false>
-__device__ void run_pass_to(const SelArgs& a, const SelState& s, u64 tile0, u64 step, PassSmem<NT>& ps, u64* cnt_a,
-                            u64* cnt_b) {
+// a to the output, b to candidate buffer s.dst, the counts on the state's.
+template <int NT, int DT>
+__device__ __forceinline__ void run_pass(const SelArgs& a, const SelState& s, u64 tile0, u64 step, PassSmem<NT>& ps) {
     typedef Key<DT> K;
     typedef typename K::raw_t raw_t;
     typedef typename K::key_t key_t;
@@ -108,35 +100,25 @@ __device__ void run_pass_to(const SelArgs& a, const SelState& s, u64 tile0, u64 
     sink.out_keys = static_cast<raw_t*>(a.out_keys);
     sink.out_idx = a.out_idx;
     sink.out_base = s.out_base;
-    sink.cap_a = a.kth_only ? 0 : s.k_rem;
+    sink.cap_a = s.k_rem;
     sink.ck = static_cast<key_t*>(a.cand_key[s.dst - 1]);
     sink.ci = a.cand_idx[s.dst - 1];
     sink.cap_b = a.cap_b;
-    sink.cnt_a = cnt_a;
-    sink.cnt_b = cnt_b;
+    sink.cnt_a = &a.st->cnt_a;
+    sink.cnt_b = &a.st->cnt_b;
     const ct lo = C::from128(s.lo), pl = C::from128(s.pl), pr = C::from128(s.pr);
-    const bool has_a = pl > lo, exact = ONLY_EXACT || lo != (ct)0;
-    if (INPUT_ONLY || s.src == SRC_INPUT) {
+    const bool has_a = pl > lo, exact = lo != (ct)0;
+    if (s.src == SRC_INPUT) {
         const InputSrc<DT> src = InputSrc<DT>::make(a.keys, s.m_src);
         if (exact) pass_tiles<NT, true, true, DT>(src, tile0, step, lo, pl, pr, sink, ps);
-        else if constexpr (!ONLY_EXACT) {
-            if (has_a) pass_tiles<NT, true, false, DT>(src, tile0, step, lo, pl, pr, sink, ps);
-            else pass_tiles<NT, false, false, DT>(src, tile0, step, lo, pl, pr, sink, ps);
-        }
-    } else if constexpr (!INPUT_ONLY) {
+        else if (has_a) pass_tiles<NT, true, false, DT>(src, tile0, step, lo, pl, pr, sink, ps);
+        else pass_tiles<NT, false, false, DT>(src, tile0, step, lo, pl, pr, sink, ps);
+    } else {
         CandSrc<KW> src{static_cast<const key_t*>(a.cand_key[s.src - 1]), a.cand_idx[s.src - 1], s.m_src};
         if (exact) pass_tiles<NT, true, true, DT>(src, tile0, step, lo, pl, pr, sink, ps);
-        else if constexpr (!ONLY_EXACT) {
-            if (has_a) pass_tiles<NT, true, false, DT>(src, tile0, step, lo, pl, pr, sink, ps);
-            else pass_tiles<NT, false, false, DT>(src, tile0, step, lo, pl, pr, sink, ps);
-        }
+        else if (has_a) pass_tiles<NT, true, false, DT>(src, tile0, step, lo, pl, pr, sink, ps);
+        else pass_tiles<NT, false, false, DT>(src, tile0, step, lo, pl, pr, sink, ps);
     }
-}
-
-template <int NT, int DT, bool INPUT_ONLY = false, bool ONLY_EXACT = false>
-__device__ __forceinline__ void run_pass(const SelArgs& a, const SelState& s, u64 tile0, u64 step,
-                                         PassSmem<NT>& ps) {
-    run_pass_to<NT, DT, INPUT_ONLY, ONLY_EXACT>(a, s, tile0, step, ps, &a.st->cnt_a, &a.st->cnt_b);
 }
 
 // ------------------------------------------------------- pickPivots
@@ -203,9 +185,10 @@ template <int DT, class SM> __device__ void plan_level(const SelArgs& a, SM& sm,
 
 // ------------------------------------------------- finish in one block
 // At most T undecided elements remain in the source: gather them, select the
-// one of rank k_rem, emit every element not above it.
+// one of rank k_rem, emit every element not above it (KTH_TOO: unless the call
+// wants the rank-k pair alone).
 
-template <int DT, class SM> __device__ void block_finish(const SelArgs& a, SM& sm) {
+template <int DT, bool KTH_TOO = false, class SM> __device__ void block_finish(const SelArgs& a, SM& sm) {
     constexpr int NT = SM::THREADS;
     typedef Key<DT> K;
     typedef typename K::raw_t raw_t;
@@ -257,10 +240,11 @@ template <int DT, class SM> __device__ void block_finish(const SelArgs& a, SM& s
         return;
     }
     const ct kth = block_select_hist<KW, NT>(sm.samp, count, lo, hi, (u32)(s.k_rem - 1), sm.hs);
-    if (threadIdx.x == 0) sm.kept = a.kth_only ? (u32)s.k_rem : 0u;
+    const bool write = !KTH_TOO || !a.kth_only;
+    if (threadIdx.x == 0) sm.kept = write ? 0u : (u32)s.k_rem;
     __syncthreads();
     raw_t* ok_out = static_cast<raw_t*>(a.out_keys);
-    for (u32 base = 0; base < count && !a.kth_only; base += NT * U) {
+    for (u32 base = 0; write && base < count; base += NT * U) {
         u32 selm = 0;
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -295,13 +279,13 @@ template <int DT, class SM> __device__ void block_finish(const SelArgs& a, SM& s
 
 
 // One recursion level run by this block alone: plan, pass, branch.
-template <int DT, bool ONLY_EXACT, class SM>
+template <int DT, class SM>
 __device__ __forceinline__ void block_level(const SelArgs& a, SM& sm) {
     SelState* g = a.st;
     plan_level<DT>(a, sm, false);
     {
         const SelState s = *g;
-        run_pass<SM::THREADS, DT, false, ONLY_EXACT>(a, s, 0, 1, sm.ps);
+        run_pass<SM::THREADS, DT>(a, s, 0, 1, sm.ps);
     }
     __syncthreads();
     if (threadIdx.x == 0) decide(*g);
@@ -310,7 +294,7 @@ __device__ __forceinline__ void block_level(const SelArgs& a, SM& sm) {
 
 // Recursion levels run by this block alone until at most T elements remain in
 // the source, then the exact finish.  Precondition: no pass pending.
-template <int DT, bool ONLY_EXACT, class SM>
+template <int DT, class SM>
 __device__ void block_levels_and_finish(const SelArgs& a, SM& sm) {
     SelState* g = a.st;
     for (u32 it = 0; it < MAX_BLOCK_LEVELS; ++it) {
@@ -318,7 +302,7 @@ __device__ void block_levels_and_finish(const SelArgs& a, SM& sm) {
             block_finish<DT>(a, sm);
             return;
         }
-        block_level<DT, ONLY_EXACT>(a, sm);
+        block_level<DT>(a, sm);
     }
     if (threadIdx.x == 0) {
         g->status = ST_EINTERNAL;

@@ -105,42 +105,6 @@ template <int DT> struct InputSrc {
         unpack(v, kk);
     }
 
-    // The keys alone (positions from idx_of); bit s of the result = valid.
-    template <int NT> __device__ __forceinline__ u32 load16_keys(u64 base, key_t (&kk)[16]) const {
-        const u32 tid = threadIdx.x;
-        const u64 ext = extent();
-        if (base + (u64)NT * 16 <= ext) {
-            const uint4* p = reinterpret_cast<const uint4*>(keys) + base / EPV;
-            uint4 v[NV];
-#pragma unroll
-            for (int j = 0; j < NV; ++j) v[j] = ld_stream(p + j * NT + tid);
-            unpack(v, kk);
-            u32 valid = 0xFFFFu;
-            if (base < head) { // the first tile: slots before the first key
-#pragma unroll
-                for (int q = 0; q < 16; ++q)
-                    if (base + (u64)((q / EPV) * NT + tid) * EPV + (q % EPV) < head) valid &= ~(1u << q);
-            }
-            return valid;
-        }
-        u32 valid = 0;
-#pragma unroll
-        for (int j = 0; j < NV; ++j) {
-#pragma unroll
-            for (int i = 0; i < EPV; ++i) {
-                const u64 e = base + (u64)(j * NT + tid) * EPV + i;
-                const int q = j * EPV + i;
-                if (e >= head && e < ext) {
-                    kk[q] = K::fwd(keys[e]);
-                    valid |= 1u << q;
-                } else {
-                    kk[q] = 0;
-                }
-            }
-        }
-        return valid;
-    }
-
     // 16 elements per thread of the tile at tile coordinate `base`: slot
     // s = j*EPV + i is tile element base + (j*NT + tid)*EPV + i.  Bit s of the
     // returned mask = valid; ii receives positions.
@@ -317,34 +281,6 @@ template <int DT> struct Sink {
             out_idx[out_base + pos] = x;
         }
     }
-    // n staged a-elements (raw keys) to output positions pos..pos+n-1 (all
-    // lanes of a warp call; coalesced)
-    template <class QK>
-    __device__ __forceinline__ void copy_a(u64 pos, const QK* sk, const u32* si, u32 n) const {
-        if (pos + n <= cap_a) {
-            raw_t* ok = out_keys + out_base + pos;
-            u32* oi = out_idx + out_base + pos;
-            for (u32 e = lane_id(); e < n; e += 32) {
-                ok[e] = (raw_t)sk[e];
-                oi[e] = si[e];
-            }
-        } else {
-            for (u32 e = lane_id(); e < n; e += 32) put_a_raw(pos + e, (raw_t)sk[e], si[e]);
-        }
-    }
-    template <class QK>
-    __device__ __forceinline__ void copy_b(u64 pos, const QK* sk, const u32* si, u32 n) const {
-        if (pos + n <= cap_b) {
-            key_t* bk = ck + pos;
-            u32* bi = ci + pos;
-            for (u32 e = lane_id(); e < n; e += 32) {
-                bk[e] = (key_t)sk[e];
-                bi[e] = si[e];
-            }
-        } else {
-            for (u32 e = lane_id(); e < n; e += 32) put_b(pos + e, (key_t)sk[e], si[e]);
-        }
-    }
     __device__ __forceinline__ void put_b(u64 pos, key_t k, u32 x) const {
         if (pos < cap_b) {
             ck[pos] = k;
@@ -359,13 +295,19 @@ template <int DT> struct Sink {
 // instead of a new sample.  The position takes only `bn` bits of the packed
 // composite, so that the bins of a bracket of few distinct keys are not spent on
 // positions that no element has.
+// COUNTS: elements are counted; KTH: the call may want the rank-k pair alone, when no
+// a element is written (batches never do, and the test cost k_batched 100 bytes of
+// spills).
 struct NoBins {
-    static constexpr bool COUNTS = false;
+    static constexpr bool COUNTS = false, KTH = false;
     template <class K> __device__ __forceinline__ void add(K, u32) const {}
+};
+struct NoBinsKth : NoBins {
+    static constexpr bool KTH = true;
 };
 template <int KW> struct BinHist {
     typedef typename Comp<KW>::t ct;
-    static constexpr bool COUNTS = true;
+    static constexpr bool COUNTS = true, KTH = true;
     u32* h;
     ct base;
     u32 sh, bn;
@@ -757,7 +699,7 @@ __device__ __forceinline__ void classify_emit(const KeyT (&kk)[16], PosF pos, u3
     u64 ra = sm.ba[warp], rb = sm.bb[warp];
     const u32 below = lanemask_lt();
     typedef typename Key<DT>::raw_t raw_t;
-    if (HAS_A && sink.cap_a != 0 && __any_sync(0xffffffffu, ma)) {
+    if (HAS_A && (!Bins::KTH || sink.cap_a != 0) && __any_sync(0xffffffffu, ma)) {
         if (ra + wa <= sink.cap_a) { // the warp's run fits: no per-element bound
             raw_t* okp = sink.out_keys + sink.out_base + ra;
             u32* oip = sink.out_idx + sink.out_base + ra;

@@ -186,7 +186,7 @@ __device__ __forceinline__ void pass_any(const Src& src, bool dense, typename Co
 // leaves the 64 registers that takes.  2^28 f32 keys at k = n / 3: 808 us a call, 1039
 // with three blocks and the bins in registers.
 template <int KW> struct SmemBins {
-    static constexpr bool COUNTS = true;
+    static constexpr bool COUNTS = true, KTH = true;
     u32 h[HB_BINS];
     BinHist<KW> b;
     __device__ __forceinline__ void add(typename Comp<KW>::key_t k, u32 x) const { b.add(k, x); }
@@ -332,8 +332,8 @@ __device__ __noinline__ void pass_again(const SelArgs& a, bool armed, HereSmem<K
     const Sink<DT> sink = make_sink<DT>(a, s);
     WarpQ<Key<DT>::KW>& q = wq[threadIdx.x >> 5];
     if (s.src == SRC_INPUT)
-        pass_any<PASS_NT, DT>(InputSrc<DT>::make(a.keys, s.m_src), s.dense != 0, lo, pl, pr, sink, ps, q, NoBins{});
-    else pass_any<PASS_NT, DT>(cand_src<DT>(a, s), s.dense != 0, lo, pl, pr, sink, ps, q, NoBins{});
+        pass_any<PASS_NT, DT>(InputSrc<DT>::make(a.keys, s.m_src), s.dense != 0, lo, pl, pr, sink, ps, q, NoBinsKth{});
+    else pass_any<PASS_NT, DT>(cand_src<DT>(a, s), s.dense != 0, lo, pl, pr, sink, ps, q, NoBinsKth{});
     pass_epilogue<Key<DT>::KW, PASS_NT, SyncBlock, false>(a, es, armed ? nullptr : &s);
 }
 
@@ -363,7 +363,7 @@ template <int DT> __global__ void __launch_bounds__(PASS_NT, Key<DT>::KW == 32 ?
         return;
     }
     pass_any<PASS_NT, DT>(cand_src<DT>(a, s), s.dense != 0, C::from128(s.lo), C::from128(s.pl), C::from128(s.pr),
-                          make_sink<DT>(a, s), ps, sm.wq[threadIdx.x >> 5], NoBins{});
+                          make_sink<DT>(a, s), ps, sm.wq[threadIdx.x >> 5], NoBinsKth{});
     pass_epilogue<KW, PASS_NT, SyncBlock, false>(a, es);
 }
 
@@ -899,7 +899,7 @@ template <int DT> __global__ void __launch_bounds__(BLK_NT) k_small(SelArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     if (threadIdx.x == 0) init_state<DT>(a.st, a);
     __syncthreads();
-    block_finish<DT>(a, *reinterpret_cast<SmallSmem<DT>*>(smem_raw));
+    block_finish<DT, true>(a, *reinterpret_cast<SmallSmem<DT>*>(smem_raw));
 }
 
 // k = 1: the minimum pair (base case of Algorithm "select");
@@ -1040,7 +1040,6 @@ static SelArgs make_args(const void* keys, u64 n, u64 k, void* out_keys, u32* ou
     a.seed = tu.seed;
     a.parts = tu.parts;
     a.sample = tu.sample;
-    a.finish_T = tu.T;
     a.z = tu.z;
     a.flags = tu.flags;
     a.aligned = (reinterpret_cast<uintptr_t>(keys) & 15u) == 0;
