@@ -263,7 +263,8 @@ topk_status topk_runs_delete_min_flexible(topk_ctx *ctx, const void *d_keys,
  * When params is NULL, or leaves block_threads, sample_size,
  * finish_threshold and split_rows all zero, rows of at most 2^19 keys whose k is
  * at most 2048 (1024 for u64), and rows of at most 4096 (2048) keys, are read
- * once by one block each and selected from a list in shared memory; for the
+ * once by one block each and selected from a list in shared memory, the longest
+ * of them only where the batch's other rows keep the GPU busy meanwhile; for the
  * others the choice remembered by topk_tune_batched for this dtype and row count
  * (power-of-two bucket) is used if there is one, else 1024 threads, a
  * 2048-element sample, the largest T and a split length of 2^15.  Settings that
@@ -344,6 +345,7 @@ topk_status topk_frequent(topk_ctx *ctx, const void *d_objects, uint64_t n, topk
  * length of 2^13, 2^15, 2^17 and none, times each with CUDA events on
  * `stream` (best of three after one warm-up), and remembers the fastest for
  * this dtype and row-count bucket (floor(log2(rows))) in the context.
+ * Every row runs by the general path, which these settings are for.
  * Arguments as topk_select_batched; every output is overwritten many times
  * (the last run uses the chosen setting, so the outputs are that call's
  * result).

@@ -320,9 +320,9 @@ template <int KW> struct PlanSmem {
 // they are more than the finish holds; returns at once otherwise, and where the window
 // was narrowed on its source (every draw has to count).
 //
-// Replaces a sampling kernel and a one-block pivot kernel that passed the
-// sample through global memory: 17 us on 2^28 f32 keys, 12 us now
-// (30 us and 16 us where most of the sample ties with the pivots).
+// 12 us on 2^28 f32 keys, 16 where most of the sample ties with the pivots; a
+// sampling kernel and a one-block pivot kernel that pass the sample through global
+// memory take 17 and 30.
 template <int DT> __global__ void __launch_bounds__(CL_NT) k_plan(SelArgs a, int first) {
     typedef Key<DT> K;
     constexpr int KW = K::KW;
@@ -476,9 +476,9 @@ template <int KW> struct FinSmem {
 // write, about twenty times at most and usually five, at 40 us for 4e6 elements
 // each.  `first`: the call's only kernel, the source is the input.
 //
-// Replaces a one-block finish that held at most 16384 elements and sampled
-// again above that: 13.0 us for 12345 keys, 11.4 us now; at the end of a
-// selection from 2^25 or more keys 11 to 20 us, 9 to 13 us now.
+// 11.4 us for 12345 keys and 9 to 13 us at the end of a selection from 2^25 or more
+// keys; one block that holds 16384 elements and samples again above that takes 13.0
+// and 11 to 20.
 template <int DT> __global__ void __launch_bounds__(CL_NT) k_finish(SelArgs a, int first) {
     grid_dep_wait();
     grid_dep_release();

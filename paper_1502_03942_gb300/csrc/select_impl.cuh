@@ -17,9 +17,9 @@
 //                        the output and the rank-k pair
 // Inputs of at most T keys take one launch: k_small (1 block) up to SMALL_MAX keys,
 // k_finish above.
-// Each recursion level used to sample anew (k_sample, k_pivots: about 17 us) before
-// its pass, two or three times a call; the bins give the second level exact
-// counts for nothing and narrow by a factor of about 1000 instead of 30.
+// k_pass also plans for itself and reads the input again after a first level that
+// failed (plan_here).  The bins give the second level exact counts for nothing and
+// narrow by a factor of about 1000; a new sample narrows by 30 and takes 17 us.
 // k = 1 (the base case of Algorithm "select", a global minimum) and k = n
 // (everything selected) take one reduction kernel instead.
 #pragma once
