@@ -267,33 +267,45 @@ template <int KW> struct RowsCfg {
 // 82 / 43; 64 rows of 2^18 59 / 66, of 2^19 101 / 88; 128 rows of 2^19 106 / 112; 64 rows
 // of 2^U(10, 18) 53 / 73; 4000 rows of 2000 keys and 4 of 2^18 107 / 387.
 struct RowsPlan {
+    enum : u32 { LEFT = 1, MID = 2, MID_LEFT = 4 }; // rows left whatever the limit; rows of 2^13 keys to the split length
     u32 longest, shortest, nshort, flags;
     u64 keys;
 };
 // The longest row that k_rows takes (0: it takes none).  All NT threads call.
 template <int KW, int NT> __device__ u32 rows_limit(const BatchArgs& b, RowsPlan& p) {
-    enum : u32 { LEFT = 1, MID = 2, MID_LEFT = 4 }; // rows left whatever the limit; rows of 2^13 keys to the split length
     if (b.row_keys || b.split == WIDE_NONE) return (u32)ROWS_MAX; // (no row is spread over the GPU)
     if (threadIdx.x == 0) p = RowsPlan{0u, 0xFFFFFFFFu, 0u, 0u, 0ull};
     __syncthreads();
     u32 mx = 0, mn = 0xFFFFFFFFu, ns = 0, fl = 0;
     u64 sum = 0;
-    for (u32 i = threadIdx.x; i < b.rows; i += NT) {
-        const u64 n = row_len(b, i), k = b.row_k[i];
-        if (k == 0 || k > n || n > 0xFFFFFFFFull) {
-            mn = 0; // (reported by whoever takes it)
-            continue;
+    constexpr int U = 4; // rows whose loads are in flight together
+    for (u32 i0 = threadIdx.x; i0 < b.rows; i0 += U * NT) {
+        u64 len[U], rank[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const u32 i = i0 + u * NT < b.rows ? i0 + u * NT : i0;
+            len[u] = row_len(b, i);
+            rank[u] = b.row_k[i];
         }
-        const bool mid = n > 8192 && n <= b.split;
-        if (n > RowsCfg<KW>::CAP && k > RowsCfg<KW>::KMAX) {
-            fl |= mid ? LEFT | MID_LEFT : LEFT;
-            continue;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (i0 + u * NT >= b.rows) continue;
+            const u64 n = len[u], k = rank[u];
+            if (k == 0 || k > n || n > 0xFFFFFFFFull) {
+                mn = 0; // (reported by whoever takes it)
+                continue;
+            }
+            const bool mid = n > 8192 && n <= b.split;
+            if (n > RowsCfg<KW>::CAP && k > RowsCfg<KW>::KMAX) {
+                fl |= mid ? RowsPlan::LEFT | RowsPlan::MID_LEFT : RowsPlan::LEFT;
+                continue;
+            }
+            fl |= (mid ? RowsPlan::MID : 0u) | (n > ROWS_MAX ? RowsPlan::LEFT : 0u);
+            ns += (u32)(n <= b.split);
+            sum += n <= ROWS_MAX ? n : 0;
+            mx = max(mx, (u32)n);
+            mn = min(mn, (u32)n);
         }
-        fl |= (mid ? MID : 0u) | (n > ROWS_MAX ? LEFT : 0u);
-        ns += (u32)(n <= b.split);
-        sum += n <= ROWS_MAX ? n : 0;
-        mx = max(mx, (u32)n);
-        mn = min(mn, (u32)n);
     }
     mx = __reduce_max_sync(0xffffffffu, mx);
     mn = __reduce_min_sync(0xffffffffu, mn);
@@ -312,9 +324,9 @@ template <int KW, int NT> __device__ u32 rows_limit(const BatchArgs& b, RowsPlan
     const u64 total = b.row_off[b.rows] - b.row_off[0];
     const bool many = p.nshort > 2 * b.sms;
     u64 limit = ROWS_MAX;
-    if ((p.flags & LEFT) || p.longest > (7ull << 14) + total / 128 + ((p.flags & MID) || many ? 1ull << 18 : 0ull)) {
+    if ((p.flags & RowsPlan::LEFT) || p.longest > (7ull << 14) + total / 128 + ((p.flags & RowsPlan::MID) || many ? 1ull << 18 : 0ull)) {
         limit = p.keys / 256 < ROWS_MAX ? p.keys / 256 : ROWS_MAX;
-        if (limit < b.split) limit = many || (p.flags & (MID | MID_LEFT)) == MID ? b.split : 0u;
+        if (limit < b.split) limit = many || (p.flags & (RowsPlan::MID | RowsPlan::MID_LEFT)) == RowsPlan::MID ? b.split : 0u;
     }
     return p.shortest <= limit ? (u32)limit : 0u;
 }
@@ -337,6 +349,11 @@ template <int KW> __global__ void __launch_bounds__(1024) k_batch_order(BatchArg
     if (limit == 0) {
         if (threadIdx.x == 0) b.words[3] = 0;
         order_rows<1024>(b, nullptr, b.rows, true);
+        return;
+    }
+    if (!b.row_keys && b.split != WIDE_NONE && !(plan.flags & RowsPlan::LEFT) && plan.longest <= limit) { // all of them
+        if (threadIdx.x == 0) b.words[3] = b.rows;
+        order_rows<1024>(b, nullptr, b.rows, false);
         return;
     }
     if (threadIdx.x == 0) nmine = nrest = 0;
